@@ -161,3 +161,27 @@ def test_full_size_residual_is_the_schur_complement_on_sampled_rows(dev):
     np.testing.assert_allclose(got, ref, rtol=0, atol=1e-4 * amax)
     # complete pivoting: |R_{k+1}| <= 2 max|R_k| = 2 |pivot_k| entrywise
     assert np.abs(got).max() <= 2 * abs(piv[-1]) + 1e-4 * amax
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64, torch.bfloat16])
+@pytest.mark.parametrize("m,n,r,pad", [(1, 1, 1, 0), (5, 1, 1, 0), (7, 3, 3, 2), (64, 5, 4, 0), (33, 66, 9, 1),
+                                       (1000, 1023, 6, 0), (511, 1024, 6, 4), (2049, 4099, 5, 0)])
+def test_flat_passes_equal_the_element_by_element_form(dev, m, n, r, pad, dtype):
+    """16-byte groups (which run over row ends when n is no multiple of the vector width) against
+    the scalar passes that a residual buffer off the 16-byte grid takes: the same bits."""
+    g = torch.Generator().manual_seed(m * 7 + n)
+    A = torch.randn((m, n + pad), generator=g, dtype=torch.float64).to(dtype).to(dev)[:, :n]
+    wide = torch.float64 if dtype == torch.float64 else torch.float32
+    out = []
+    for off in (0, 1):
+        buf = torch.full((m * n + 1,), float("nan"), dtype=wide, device=dev)
+        R = buf[off:off + m * n].view(m, n)
+        I = torch.empty(r, dtype=torch.int32, device=dev)
+        J = torch.empty(r, dtype=torch.int32, device=dev)
+        piv = torch.empty(r, dtype=torch.float64, device=dev)
+        with cur.Handle(m, n, r, cur.CUR_F32) as hd:
+            cur.cur_aca_full(hd.h, A, r, R, I, J, piv)
+            st = cur.cur_sync_status(hd.h)
+        out.append((st, I.tolist(), J.tolist(), piv.tolist(), R.clone()))
+    assert out[0][:4] == out[1][:4] and out[0][0] == cur.CUR_OK
+    assert torch.equal(out[0][4], out[1][4])

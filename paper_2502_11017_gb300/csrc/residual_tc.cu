@@ -9,22 +9,31 @@
 // N = 128 columns, K = r) the C panel is the MMA's A operand, read from tensor memory,
 // and the tile's W^T the B operand, read from shared memory; a TMEM lane is a row of A.
 //
-// Per CTA (persistent, one per SM, 608 threads; its tiles run along row panels):
-//   TMEM         two accumulators (128 columns each) and two C panels (hi in 64
-//                columns, lo in the next 64): the next panel is split and stored while
-//                the current one is in use
+// A unit of work is one W^T tile (r x 128, hi and lo: 64 KB at r = 64, as much as the A tile it
+// serves) and a pair of row panels (pw = 2; 1 where that would leave SMs idle): 1.5 bytes
+// through L2 per byte of A instead of 2. What bounds the kernel is A's latency: 96 KB of A in
+// flight per SM (what the two W stages leave) come back after ~3.8 us under load, 477 us at
+// 65536 x 8192 (0.66 of the copy rate); neither the MMAs (0.31 of the time), their issue, nor
+// the epilogue's arithmetic showed in the time when they were shortened.
+//
+// Per CTA (persistent, one per SM, 608 threads; its units run along the panels):
+//   TMEM         two accumulators (128 columns each) and the unit's two C panels (hi in 64
+//                columns, lo in the next 64)
 //   warp 0       TMA producer of W^T (128 columns of A x r, hi and lo, 128-byte swizzle,
-//                K-major) into two stages, so the next tile's W loads during this one's MMAs
+//                K-major) into two stages, so the next unit's W loads during this one's MMAs
 //   warp 1       MMA issuer (one thread): 3 passes x r/8 MMAs per tile into one of the
 //                two accumulators
-//   warp 18      TMA producer of A: 32-row x 128-column sub-tiles (16 KB, four 32 x 32
-//                boxes with 128-byte swizzle) into a ring of up to 10 slots; A is read
-//                from HBM exactly once
+//   warp 18      TMA producer of A: sub-tiles of 32 rows x 64 columns (8 KB, two 32 x 32
+//                boxes with 128-byte swizzle) into a ring of nq slots per lane quarter; A is
+//                read from HBM exactly once. Every warp of a quarter waits for every sub-tile
+//                of its ring in order, also those it does not read: with one ring for all
+//                quarters a warp skipped phases of a slot, and the parity of the phase two
+//                before passed for its own (sum A^2 then differed from run to run)
 //   warps 2..17  epilogue: warp (lane quarter q, column group g) reads its 32 rows x 32
-//                accumulator columns with tcgen05.ld and the same block of A from shared
-//                memory (16-byte loads, conflict-free through the swizzle), and folds
-//                max|E|, sum E^2, sum A^2; the same warps split C rows into TF32 hi and
-//                lo and store them into TMEM with tcgen05.st when a panel begins
+//                accumulator columns with tcgen05.ld, hands the accumulator back, reads the
+//                same block of A from shared memory (16-byte loads, conflict-free through
+//                the swizzle), and folds max|E|, sum E^2, sum A^2; the same warps split C
+//                rows into TF32 hi and lo and store them with tcgen05.st
 // Out-of-range rows and columns read as zeros from every operand (TMA fill; zero C rows),
 // so E = 0 there and no element needs a mask.
 // Waits are bounded; on a timeout the CTA records CUR_ERR_TIMEOUT, waits (bounded) for
@@ -112,8 +121,8 @@ __global__ void __launch_bounds__(256) tc_prep_w(const double* __restrict__ U, c
 
 constexpr int kAR = 32;                     // rows of A per staged sub-tile (one lane quarter)
 constexpr int kABox = kAR * 32 * 4;         // 4 KB: 32 rows x 32 columns FP32, 128-byte swizzle
-constexpr int kASub = 4 * kABox;            // 16 KB: 32 rows x 128 columns
-constexpr int kNAMax = 10;                  // A ring slots at most
+constexpr int kASub = 2 * kABox;            // 8 KB: 32 rows x 64 columns
+constexpr int kNQMax = 5;                   // A ring slots per lane quarter at most
 constexpr int kEpiWarps = 16;               // epilogue: 4 lane quarters x 4 column groups
 constexpr int kTmemCols = 512;              // accumulators at 0 and 128, C panels at 256 and 384
 constexpr int kCLo = 64;                    // TMEM column offset of a panel's lo words
@@ -121,8 +130,9 @@ constexpr int kCLo = 64;                    // TMEM column offset of a panel's l
 struct TcArgs {
     int64_t m, n;
     const float* C;   // m x r, row-major
-    int r, nch, ksteps, na;
-    int64_t ntile_n, ntiles;
+    int r, nch, ksteps, nq;
+    int64_t ntile_n, npanels, units;
+    int pw;         // row panels per unit (1 or 2)
     double* part;   // 4 doubles per CTA
     int* status;
 };
@@ -167,37 +177,62 @@ __device__ __forceinline__ void store_c_panel(const TcArgs& a, int64_t panel, ui
     tc_fence_before();
 }
 
+// Adds a tile's FP32 sum to a running one: as a double-float (exact to ~2^-48, five FP32
+// operations; in FP64 the two sums of 512 threads took a quarter of the FP64 pipe's time per
+// tile, all on the epilogue's critical path), or in FP64 where its range is needed.
+__device__ __forceinline__ void tc_sum(float x, double& wide, df64& acc) {
+    if (x < 1e28f) {
+        const df64 t = two_sum(acc.h, x);
+        acc = df64{t.h, __fadd_rn(acc.l, t.l)};
+    } else {
+        wide += (double)x;
+    }
+}
+
+// The tiles of one CTA in order: fn(unit, panel group, column tile, panel of the group).
+template <typename F>
+__device__ __forceinline__ void tc_tiles(const TcArgs& a, F&& fn) {
+    const int64_t G = gridDim.x;
+    const int64_t u0 = a.units * blockIdx.x / G, u1 = a.units * (blockIdx.x + 1) / G;
+    int64_t pg = u0 / a.ntile_n, ct = u0 - pg * a.ntile_n;
+    for (int64_t u = u0; u < u1; ++u) {
+        const int np = (int)min((int64_t)a.pw, a.npanels - pg * a.pw);
+        for (int hp = 0; hp < np; ++hp)
+            if (!fn(u - u0, pg, ct, hp, np)) return;
+        if (++ct == a.ntile_n) { ct = 0; ++pg; }
+    }
+}
+
 __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ CUtensorMap mWh,
                                                         const __grid_constant__ CUtensorMap mWl,
                                                         const __grid_constant__ CUtensorMap mA,
                                                         TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int nch = a.nch, na = a.na;
+    const int nch = a.nch, nq = a.nq;
     const uint32_t half_bytes = (uint32_t)nch * kChunk;   // W^T hi (or lo) of one tile
     unsigned char* WB = sm;                     // 2 stages x (hi, lo)
-    unsigned char* AS = WB + 4 * (size_t)half_bytes;   // ring of na A sub-tiles
-    __shared__ __align__(8) uint64_t wfull[2], wempty[2], cfull[2], accf[2], acce[2], af[kNAMax], ae[kNAMax];
+    unsigned char* AS = WB + 4 * (size_t)half_bytes;   // four rings of nq A sub-tiles
+    __shared__ __align__(8) uint64_t wfull[2], wempty[2], cfull, accf[2], acce[2], af[4 * kNQMax],
+        ae[4 * kNQMax];
     __shared__ uint32_t tslot;
-    __shared__ int abort_flag;
+    __shared__ volatile int abort_flag;
     __shared__ double rmx[kEpiWarps], rse[kEpiWarps], rsa[kEpiWarps];
     __shared__ int rbad[kEpiWarps];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t G = gridDim.x;
-    const int64_t t0 = a.ntiles * blockIdx.x / G, t1 = a.ntiles * (blockIdx.x + 1) / G;
 
     if (tid == 0) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(&wfull[s], 1);
             mbar_init(&wempty[s], 1);
-            mbar_init(&cfull[s], kEpiWarps);
             mbar_init(&accf[s], 1);
             mbar_init(&acce[s], kEpiWarps);
         }
-        for (int s = 0; s < na; ++s) {
+        for (int s = 0; s < 4 * nq; ++s) {
             mbar_init(&af[s], 1);
             mbar_init(&ae[s], 4);   // the four column-group warps of one lane quarter
         }
+        mbar_init(&cfull, kEpiWarps);
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -210,20 +245,23 @@ __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ 
     if (warp == 0) {
         // ------------------------------------------------------------ W^T producer
         if (lane == 0) {
-            int64_t nw = 0;   // tiles whose W was issued
+            int64_t nw = 0;   // units whose W was issued
             bool ok = true;
-            for (int64_t t = t0; t < t1 && !abort_flag; ++t, ++nw) {
-                const int64_t ct = t % a.ntile_n;
+            tc_tiles(a, [&](int64_t, int64_t, int64_t ct, int hp, int) {
+                if (abort_flag) return false;
+                if (hp > 0) return true;
                 const int s = (int)(nw & 1);
                 const int64_t u = nw >> 1;
-                if (u > 0 && !mbar_wait(&wempty[s], (uint32_t)((u - 1) & 1))) { ok = false; break; }
+                if (u > 0 && !mbar_wait(&wempty[s], (uint32_t)((u - 1) & 1))) { ok = false; return false; }
                 unsigned char* dst = WB + (size_t)s * 2 * half_bytes;
                 mbar_expect_tx(&wfull[s], 2 * half_bytes);
                 for (int c = 0; c < nch; ++c) {
                     tma_load_2d(dst + c * kChunk, &mWh, &wfull[s], 32 * c, (int)(ct * kTcBN));
                     tma_load_2d(dst + half_bytes + c * kChunk, &mWl, &wfull[s], 32 * c, (int)(ct * kTcBN));
                 }
-            }
+                ++nw;
+                return true;
+            });
             if (!ok) { abort_flag = 1; set_status(a.status, CUR_ERR_TIMEOUT); }
             // after an abort, wait (bounded) for the last copy into each stage: the MMA
             // warp consumed every full barrier otherwise
@@ -234,39 +272,47 @@ __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ 
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_tf32(kTcBM, kTcBN);
-            int64_t cur_panel = -1, pc = -1, it = 0;
+            int64_t cur = -1, pc = 0, it = 0;
             bool ok = true;
+            const int ksteps = a.ksteps;
             uint64_t* last_bar = nullptr;   // the barrier of the last commit and its phase
             uint32_t last_par = 0;
-            for (int64_t t = t0; t < t1 && !abort_flag; ++t, ++it) {
-                const int64_t panel = t / a.ntile_n;
-                if (panel != cur_panel) {
+            tc_tiles(a, [&](int64_t un, int64_t pg, int64_t, int hp, int np) {
+                if (abort_flag) return false;
+                if (pg != cur) {
+                    cur = pg;
+                    if (!mbar_wait(&cfull, (uint32_t)(pc & 1))) { ok = false; return false; }
                     ++pc;
-                    cur_panel = panel;
-                    if (!mbar_wait(&cfull[pc & 1], (uint32_t)((pc >> 1) & 1))) { ok = false; break; }
                 }
-                const int b = (int)(it & 1);
+                const int b = (int)(it & 1), ws = (int)(un & 1);
                 const int64_t u = it >> 1;
-                if (u > 0 && !mbar_wait(&acce[b], (uint32_t)((u - 1) & 1))) { ok = false; break; }
-                if (!mbar_wait(&wfull[b], (uint32_t)(u & 1))) { ok = false; break; }
+                if (u > 0 && !mbar_wait(&acce[b], (uint32_t)((u - 1) & 1))) { ok = false; return false; }
+                if (hp == 0 && !mbar_wait(&wfull[ws], (uint32_t)((un >> 1) & 1))) { ok = false; return false; }
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(b * kTcBN);
-                const uint32_t cpan = tmem + 256u + (uint32_t)((pc & 1) * 128);
-                const uint32_t wh = su32(WB + (size_t)b * 2 * half_bytes), wl = wh + half_bytes;
-                // Ch Wh, Cl Wh, Ch Wl
-                for (int pass = 0; pass < 3; ++pass) {
-                    const uint32_t aop = cpan + (pass == 1 ? (uint32_t)kCLo : 0u);
-                    const uint32_t bop = pass == 2 ? wl : wh;
-                    for (int k = 0; k < a.ksteps; ++k) {
-                        const uint32_t off = (uint32_t)((k >> 2) * kChunk + (k & 3) * 32);
-                        mma_tf32_ts(d, aop + (uint32_t)(8 * k), sdesc_k128(bop + off), idesc, (pass | k) != 0);
-                    }
-                }
-                mma_commit(&wempty[b]);
+                const uint32_t cpan = tmem + 256u + (uint32_t)(hp * 128);
+                const uint64_t wh = sdesc_k128(su32(WB + (size_t)ws * 2 * half_bytes));
+                const uint64_t wl = wh + (uint64_t)(half_bytes >> 4);
+                // Ch Wh, Cl Wh, Ch Wl; unrolled (r is 32 or 64: 4 or 8 steps of 8), so that a
+                // descriptor is one addition: formed in a loop, each took this one thread
+                // longer than the MMA it issued
+                auto product = [&](uint32_t aop, uint64_t bop, bool first) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        if (k < ksteps)
+                            mma_tf32_ts(d, aop + (uint32_t)(8 * k), bop + (uint64_t)(((k >> 2) * kChunk + (k & 3) * 32) >> 4),
+                                        idesc, !(first && k == 0));
+                };
+                product(cpan, wh, true);
+                product(cpan + (uint32_t)kCLo, wh, false);
+                product(cpan, wl, false);
+                if (hp == np - 1) mma_commit(&wempty[ws]);
                 mma_commit(&accf[b]);
                 last_bar = &accf[b];
                 last_par = (uint32_t)(u & 1);
-            }
+                ++it;
+                return true;
+            });
             if (!ok) { abort_flag = 1; set_status(a.status, CUR_ERR_TIMEOUT); }
             // every MMA issued has finished once the last commit has arrived
             if (last_bar) mbar_wait(last_bar, last_par);
@@ -274,24 +320,31 @@ __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ 
     } else if (warp == 2 + kEpiWarps) {
         // ------------------------------------------------------------ A producer
         if (lane == 0) {
-            int64_t idx = 0;
+            int64_t seq = 0;   // sub-tiles issued into each quarter's ring
+            int done_q = 0;    // quarters of the last sequence number issued before a timeout
             bool ok = true;
-            for (int64_t t = t0; t < t1 && ok && !abort_flag; ++t) {
-                const int64_t panel = t / a.ntile_n, ct = t - panel * a.ntile_n;
-                for (int k = 0; k < kTcBM / kAR; ++k, ++idx) {
-                    const int slot = (int)(idx % na);
-                    const int64_t use = idx / na;
-                    if (use > 0 && !mbar_wait(&ae[slot], (uint32_t)((use - 1) & 1))) { ok = false; break; }
-                    mbar_expect_tx(&af[slot], (uint32_t)kASub);
-                    for (int g = 0; g < 4; ++g)
-                        tma_load_2d(AS + (size_t)slot * kASub + g * kABox, &mA, &af[slot],
-                                    (int)(ct * kTcBN + 32 * g), (int)(panel * kTcBM + kAR * k));
+            tc_tiles(a, [&](int64_t, int64_t pg, int64_t ct, int hp, int) {
+                if (abort_flag) return false;
+                const int64_t row0 = (pg * a.pw + hp) * kTcBM;
+                for (int half = 0; half < 2; ++half, ++seq) {
+                    const int slot = (int)(seq % nq);
+                    const int64_t use = seq / nq;
+                    for (int q = 0; q < 4; ++q) {
+                        const int s = q * nq + slot;
+                        if (use > 0 && !mbar_wait(&ae[s], (uint32_t)((use - 1) & 1))) { ok = false; done_q = q; return false; }
+                        mbar_expect_tx(&af[s], (uint32_t)kASub);
+                        for (int x = 0; x < 2; ++x)
+                            tma_load_2d(AS + (size_t)s * kASub + x * kABox, &mA, &af[s],
+                                        (int)(ct * kTcBN + 64 * half + 32 * x), (int)(row0 + kAR * q));
+                    }
                 }
-            }
+                return true;
+            });
             if (!ok) { abort_flag = 1; set_status(a.status, CUR_ERR_TIMEOUT); }
-            if (abort_flag)
-                for (int64_t q = idx - 1; q >= 0 && q >= idx - na; --q)
-                    mbar_wait(&af[q % na], (uint32_t)((q / na) & 1));
+            if (abort_flag)   // every copy issued has landed (bounded waits) before the CTA ends
+                for (int q = 0; q < 4; ++q)
+                    for (int64_t x = seq - 1 + (q < done_q); x >= 0 && x >= seq + (q < done_q) - nq; --x)
+                        mbar_wait(&af[q * nq + x % nq], (uint32_t)((x / nq) & 1));
         }
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..17)
@@ -301,79 +354,70 @@ __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ 
         const uint32_t trow = (uint32_t)(32 * q) << 16;
         float mx = 0.f;
         double se = 0.0, sa = 0.0;
+        df64 sef{0.f, 0.f}, saf{0.f, 0.f};
         int bad = 0;
-        if (t0 < t1) {
-            // the first two panels; later ones are stored when the panel before them begins
-            const int64_t p0 = t0 / a.ntile_n, plast = (t1 - 1) / a.ntile_n;
-            store_c_panel(a, p0, trow, 256u, q, g, lane);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&cfull[0]);
-            if (plast > p0) {
-                store_c_panel(a, p0 + 1, trow, 384u, q, g, lane);
+        int64_t it = 0, seq = 0, cur = -1;
+        tc_tiles(a, [&](int64_t, int64_t pg, int64_t, int, int np) {
+            if (pg != cur) {
+                // every MMA of the panels before has completed (this warp has waited for the
+                // last accumulator), so their TMEM columns take the new ones
+                cur = pg;
+                for (int x = 0; x < np; ++x) store_c_panel(a, pg * a.pw + x, trow, 256u + 128u * (uint32_t)x, q, g, lane);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&cfull[1]);
+                if (lane == 0) mbar_arrive(&cfull);
             }
-        }
-        int64_t it = 0, cur_panel = -1, pc = -1;
-        const int64_t plast = t1 > t0 ? (t1 - 1) / a.ntile_n : -1;
-        for (int64_t t = t0; t < t1; ++t, ++it) {
-            const int64_t panel = t / a.ntile_n;
-            const bool fresh = panel != cur_panel;
-            if (fresh) { ++pc; cur_panel = panel; }
             const int b = (int)(it & 1);
             if (!mbar_wait(&accf[b], (uint32_t)((it >> 1) & 1))) {
                 abort_flag = 1;
                 set_status(a.status, CUR_ERR_TIMEOUT);
-                break;
-            }
-            tc_fence_after();
-            if (fresh && pc >= 1 && panel + 1 <= plast) {
-                // every MMA of the panel before this one has completed (this tile's commit
-                // follows them), so its TMEM columns take the panel after this one
-                store_c_panel(a, panel + 1, trow, 256u + (uint32_t)(((pc + 1) & 1) * 128), q, g, lane);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&cfull[(pc + 1) & 1]);
-            }
-            const int64_t idx = 4 * it + q;
-            const int slot = (int)(idx % na);
-            if (!mbar_wait(&af[slot], (uint32_t)((idx / na) & 1))) {
-                abort_flag = 1;
-                set_status(a.status, CUR_ERR_TIMEOUT);
-                break;
             }
             __syncwarp();
-            // the 32 x 32 block: accumulator columns b*128 + 32 g .. + 31 of this warp's
-            // lanes, and row `lane` of A box g (16-byte chunk c stored at c ^ (lane & 7))
-            float dall[32];
-            tmem_ld32(tmem + trow + (uint32_t)(b * kTcBN + 32 * g), dall);
-            const unsigned char* arow = AS + (size_t)slot * kASub + g * kABox + lane * 128;
+            tc_fence_after();
+            float d[32];
+            tmem_ld32(tmem + trow + (uint32_t)(b * kTcBN + 32 * g), d);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acce[b]);   // the accumulator is in registers
             // four independent chains per sum; a NaN anywhere makes the group's sum of
             // squares NaN (fmaxf alone would drop it)
             float m4[4] = {0.f, 0.f, 0.f, 0.f}, s4[4] = {0.f, 0.f, 0.f, 0.f}, a4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float4 x4 = *reinterpret_cast<const float4*>(arow + ((c ^ (lane & 7)) << 4));
-                const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float e = xs[i] - dall[4 * c + i];
-                    m4[i] = fmaxf(m4[i], fabsf(e));
-                    s4[i] = fmaf(e, e, s4[i]);
-                    a4[i] = fmaf(xs[i], xs[i], a4[i]);
+            for (int half = 0; half < 2; ++half, ++seq) {
+                const int s = q * nq + (int)(seq % nq);
+                if (!mbar_wait(&af[s], (uint32_t)((seq / nq) & 1))) {
+                    abort_flag = 1;
+                    set_status(a.status, CUR_ERR_TIMEOUT);
                 }
+                __syncwarp();
+                if (half == (g >> 1)) {
+                    // row `lane` of this warp's box (16-byte chunk c at c ^ (lane & 7))
+                    const unsigned char* arow = AS + (size_t)s * kASub + (g & 1) * kABox + lane * 128;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const float4 x4 = *reinterpret_cast<const float4*>(arow + ((c ^ (lane & 7)) << 4));
+                        const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float e = xs[i] - d[4 * c + i];
+                            m4[i] = fmaxf(m4[i], fabsf(e));
+                            s4[i] = fmaf(e, e, s4[i]);
+                            a4[i] = fmaf(xs[i], xs[i], a4[i]);
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (lane == 0) mbar_arrive(&ae[s]);
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&ae[slot]);
             const float gs = (s4[0] + s4[1]) + (s4[2] + s4[3]);
             if (gs != gs) bad = 1;
             mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
-            se += (double)gs;
-            sa += (double)((a4[0] + a4[1]) + (a4[2] + a4[3]));
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acce[b]);
-            if (abort_flag) break;
-        }
+            tc_sum(gs, se, sef);
+            tc_sum((a4[0] + a4[1]) + (a4[2] + a4[3]), sa, saf);
+            ++it;
+            return __all_sync(0xffffffffu, abort_flag == 0) != 0;
+        });
+        se += df_to_d(sef);
+        sa += df_to_d(saf);
         // reduce over the epilogue threads
         double dmx = mx;
         for (int o = 16; o > 0; o >>= 1) {
@@ -512,16 +556,19 @@ cur_status residual_tc_impl(cur_handle* h, const cur_mat* Am, const void* C, con
     a.nch = nch;
     a.ksteps = (r + 7) / 8;
     a.ntile_n = (n + kTcBN - 1) / kTcBN;
-    a.ntiles = ((m + kTcBM - 1) / kTcBM) * a.ntile_n;
+    a.npanels = (m + kTcBM - 1) / kTcBM;
+    // pairs of panels share a W^T tile once every SM has several tiles anyway
+    a.pw = a.npanels * a.ntile_n >= 8LL * G ? 2 : 1;
+    a.units = (a.npanels + a.pw - 1) / a.pw * a.ntile_n;
     a.part = part;
     a.status = h->status;
-    const int grid = (int)std::min<int64_t>(G, a.ntiles);
-    // two stages of the W^T tile (hi and lo each), then as many 16 KB A slots as fit
+    const int grid = (int)std::min<int64_t>(G, a.units);
+    // two stages of the W^T tile (hi and lo each), then as many 8 KB A slots per quarter as fit
     const size_t fixed = (size_t)4 * nch * kChunk + 1024;
     const size_t budget = 225 * 1024;
-    a.na = (int)std::min<size_t>(kNAMax, (budget - fixed) / kASub);
-    if (a.na < 4) return CUR_ERR_ARG;
-    const size_t sm = fixed + (size_t)a.na * kASub;
+    a.nq = (int)std::min<size_t>(kNQMax, (budget - fixed) / (4 * kASub));
+    if (a.nq < 2) return CUR_ERR_ARG;
+    const size_t sm = fixed + (size_t)4 * a.nq * kASub;
     CUR_TRY(smem_attr((const void*)residual_tc_k, sm));
     residual_tc_k<<<grid, 32 * (3 + kEpiWarps), sm, st>>>(mWh, mWl, mA, a);
     CUR_CK(cudaGetLastError());

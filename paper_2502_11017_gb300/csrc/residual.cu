@@ -332,6 +332,241 @@ __global__ void __launch_bounds__(256, 2) residual_k(const TA* __restrict__ A, i
     }
 }
 
+// ---- the same residual for FP32 and BF16 data at the FP32 FMA rate
+//
+// Every element is the FP32 FMA chain over k of residual_k and every 8 x 8 group of a tile folds
+// the same 64 elements in the same order, so max|E| and the tile sums are bit-identical to it.
+// What bounds it is the FMA pipe: m n r FMAs, 14.7 ms at 262144 x 16384, r = 128 (residual_k
+// took 77.6 ms: it staged W with plain loads between barriers, one CTA per SM at r = 128, so
+// that the loads, the FMAs and the reads of A followed one another). Here
+//   * two CTAs per SM: one CTA's reads of A and its partial sums run under the other's FMAs;
+//   * W comes by cp.async in chunks of 32 k, two stages, during the chunk before;
+//   * a thread has two of residual_k's groups, 16 rows x 8 columns, and its FMAs are pairs
+//     (fma.rn.f32x2, each half rounded as fmaf) of two rows of C times one column of W: per k
+//     64 of them for 4 + 4 loads from shared memory. (With 8 x 8 per thread and W stored
+//     twice over for ready pairs, 2 + 4 16-byte loads per 32 pairs, the loads took 1.2 times
+//     the FMAs' time: 28.5 ms.)
+//   * CTAs walk contiguous ranges of tiles along row panels and keep the C panel.
+constexpr int kRfB = 128;    // rows and columns of a tile; 8 x 16 threads, 16 x 8 each
+constexpr int kRfKC = 32;    // k per stage of W
+constexpr int kRfT = 128;    // threads
+
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t twice(float x) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+    return d;
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// W = U R summed in FP64 (one chain over l) and rounded to FP32 as residual_w_k does, rows of
+// npad columns, zeros past n. A block takes 32 columns and kRfWK rows k; a thread 4 k x 2 j
+// (eight FP64 chains; the FP64 pipe bounds it: r^2 n DFMAs).
+constexpr int kRfWK = 64;
+template <typename TA>
+__global__ void __launch_bounds__(256) residual_w2_k(const double* __restrict__ U, const TA* __restrict__ R, int r,
+                                                     int64_t n, int64_t npad, float* __restrict__ W) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* Us = reinterpret_cast<double*>(smem_raw);   // Us[l * 64 + k] = U(k0 + k, l)
+    double* Rs = Us + (size_t)r * kRfWK;                // Rs[l * 32 + jj] = R(l, j0 + jj)
+    const int64_t j0 = (int64_t)blockIdx.x * 32;
+    const int k0 = blockIdx.y * kRfWK;
+    for (int e = threadIdx.x; e < r * kRfWK; e += blockDim.x) {
+        const int k = e / r, l = e - k * r;
+        Us[l * kRfWK + k] = k0 + k < r ? U[(int64_t)(k0 + k) * r + l] : 0.0;
+    }
+    for (int e = threadIdx.x; e < r * 32; e += blockDim.x) {
+        const int l = e >> 5, jj = e & 31;
+        Rs[e] = j0 + jj < n ? to_d(R[(int64_t)l * n + j0 + jj]) : 0.0;
+    }
+    __syncthreads();
+    const int jg = threadIdx.x & 15, kg = threadIdx.x >> 4;
+    double acc[4][2] = {};
+    for (int l = 0; l < r; ++l) {
+        const double2 ua = *reinterpret_cast<const double2*>(Us + l * kRfWK + 4 * kg);
+        const double2 ub = *reinterpret_cast<const double2*>(Us + l * kRfWK + 4 * kg + 2);
+        const double2 rr = *reinterpret_cast<const double2*>(Rs + l * 32 + 2 * jg);
+        const double u4[4] = {ua.x, ua.y, ub.x, ub.y};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc[i][0] = fma(u4[i], rr.x, acc[i][0]);
+            acc[i][1] = fma(u4[i], rr.y, acc[i][1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = k0 + 4 * kg + i;
+        const int64_t j = j0 + 2 * jg;
+        if (k >= r || j >= npad) continue;
+        const float a = j < n ? (float)acc[i][0] : 0.f, b = j + 1 < n ? (float)acc[i][1] : 0.f;
+        *reinterpret_cast<float2*>(W + (int64_t)k * npad + j) = make_float2(a, b);
+    }
+}
+
+template <typename TA>
+__global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__ A, int64_t m, int64_t n, int64_t ld,
+                                                          const TA* __restrict__ C, const float* __restrict__ W,
+                                                          int64_t npad, int r, int64_t ntile_n, int64_t ntiles,
+                                                          double* __restrict__ part, int pairs) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* Ws = reinterpret_cast<float*>(smem_raw);   // two stages of kRfKC x 128
+    float* Ct = Ws + 2 * kRfKC * kRfB;                // r x 128 (transposed C panel)
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
+    const int64_t t0 = ntiles * blockIdx.x / gridDim.x, t1 = ntiles * (blockIdx.x + 1) / gridDim.x;
+    const int nchunk = (r + kRfKC - 1) / kRfKC;
+    double mx = 0.0, se = 0.0, sa = 0.0;
+    int bad = 0;
+    // chunk c of the column tile ct into stage s: row k is 512 bytes, one warp's 16-byte copies
+    auto load = [&](int64_t ct, int c, int s) {
+        const float* src = W + ct * kRfB + 4 * lane;
+#pragma unroll
+        for (int x = 0; x < kRfKC / 4; ++x) {
+            const int kk = 4 * x + warp, k = c * kRfKC + kk;
+            if (k < r) cp_async16(Ws + (s * kRfKC + kk) * kRfB + 4 * lane, src + (int64_t)k * npad);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int64_t panel = -1;
+    int stage = 0;
+    if (t0 < t1) load(t0 % ntile_n, 0, 0);
+    for (int64_t t = t0; t < t1; ++t) {
+        const int64_t pn = t / ntile_n, ct = t - pn * ntile_n;
+        const int64_t r0 = pn * kRfB, c0 = ct * kRfB;
+        if (pn != panel) {
+            panel = pn;
+            __syncthreads();
+            for (int e = tid; e < kRfB * r; e += kRfT) {
+                const int k = e / kRfB, i = e - k * kRfB;
+                Ct[e] = r0 + i < m ? to_f(C[(r0 + i) * r + k]) : 0.f;
+            }
+        }
+        uint64_t acc[8][8];   // rows 2 a, 2 a + 1 of the thread's sixteen, column b
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) acc[a][b] = 0ull;
+        for (int c = 0; c < nchunk; ++c, stage ^= 1) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();   // this chunk has landed, and the other stage has been read
+            if (c + 1 < nchunk) load(ct, c + 1, stage ^ 1);
+            else if (t + 1 < t1) load((t + 1) % ntile_n, 0, stage ^ 1);
+            const float* ws = Ws + stage * kRfKC * kRfB + 2 * tx;
+            const float* cs = Ct + c * kRfKC * kRfB + 16 * ty;
+            const int kc = min(kRfKC, r - c * kRfKC);
+            // operands of the next k are loaded before the FMAs of this one
+            ulonglong2 x[4], xn[4];
+            float2 y[4], yn[4];
+            auto fetch = [&](int kk, ulonglong2* xx, float2* yy) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) xx[q] = *reinterpret_cast<const ulonglong2*>(cs + kk * kRfB + 4 * q);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) yy[q] = *reinterpret_cast<const float2*>(ws + kk * kRfB + 32 * q);
+            };
+            auto step = [&](const ulonglong2* xx, const float2* yy) {
+#pragma unroll
+                for (int b = 0; b < 8; ++b) {
+                    const uint64_t w = twice(b & 1 ? yy[b >> 1].y : yy[b >> 1].x);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        fma2(acc[2 * q][b], xx[q].x, w);
+                        fma2(acc[2 * q + 1][b], xx[q].y, w);
+                    }
+                }
+            };
+            fetch(0, x, y);
+            int kk = 0;
+            for (; kk + 2 <= kc; kk += 2) {
+                fetch(kk + 1, xn, yn);
+                step(x, y);
+                fetch(min(kk + 2, kc - 1), x, y);
+                step(xn, yn);
+            }
+            if (kk < kc) step(x, y);
+        }
+        const bool whole = c0 + kRfB <= n && pairs;
+#pragma unroll
+        for (int grp = 0; grp < 2; ++grp) {
+            float tmx = 0.f, tse = 0.f, tsa = 0.f;
+            auto fold = [&](float av, float d) {
+                const float e = av - d;
+                if (!(fabsf(e) <= INFINITY)) bad = 1;
+                tmx = fmaxf(tmx, fabsf(e));
+                tse = fmaf(e, e, tse);
+                tsa = fmaf(av, av, tsa);
+            };
+#pragma unroll
+            for (int a0 = 0; a0 < 8; a0 += 4) {
+                const int64_t i0 = r0 + ty * 16 + grp * 8 + a0;
+                if (whole && i0 + 4 <= m) {   // two elements per load, sixteen loads in flight
+                    uint64_t raw[4][4];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            const TA* p = A + (i0 + a) * ld + c0 + 2 * tx + 32 * b;
+                            if constexpr (sizeof(TA) == 4)
+                                raw[a][b] = __ldcs(reinterpret_cast<const unsigned long long*>(p));
+                            else
+                                raw[a][b] = __ldcs(reinterpret_cast<const unsigned*>(p));
+                        }
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b < 8; ++b) {
+                            const uint64_t v = raw[a][b >> 1];
+                            const uint32_t bits = sizeof(TA) == 4 ? (uint32_t)(b & 1 ? v >> 32 : v)
+                                                                  : (b & 1 ? (uint32_t)v & 0xffff0000u : (uint32_t)v << 16);
+                            const int row = grp * 8 + a0 + a;
+                            const uint64_t d = acc[row >> 1][b];
+                            fold(__uint_as_float(bits), __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)));
+                        }
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        if (i0 + a >= m) break;
+#pragma unroll
+                        for (int b = 0; b < 8; ++b) {
+                            const int64_t col = c0 + 2 * tx + 32 * (b >> 1) + (b & 1);
+                            const int row = grp * 8 + a0 + a;
+                            const uint64_t d = acc[row >> 1][b];
+                            if (col < n) fold(to_f(A[(i0 + a) * ld + col]), __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)));
+                        }
+                    }
+                }
+            }
+            mx = fmax(mx, (double)tmx);
+            se += (double)tse;
+            sa += (double)tsa;
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __shared__ double rmx[kRfT / 32], rse[kRfT / 32], rsa[kRfT / 32];
+    __shared__ int rbad;
+    if (tid == 0) rbad = 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        se += __shfl_xor_sync(0xffffffffu, se, o);
+        sa += __shfl_xor_sync(0xffffffffu, sa, o);
+    }
+    __syncthreads();
+    if (bad) rbad = 1;
+    if (lane == 0) { rmx[warp] = mx; rse[warp] = se; rsa[warp] = sa; }
+    __syncthreads();
+    if (tid == 0) {
+        double a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        for (int w = 0; w < kRfT / 32; ++w) { a1 = fmax(a1, rmx[w]); a2 += rse[w]; a3 += rsa[w]; }
+        part[(int64_t)blockIdx.x * 4 + 0] = a1;
+        part[(int64_t)blockIdx.x * 4 + 1] = a2;
+        part[(int64_t)blockIdx.x * 4 + 2] = a3;
+        part[(int64_t)blockIdx.x * 4 + 3] = rbad ? 1.0 : 0.0;
+    }
+}
+
 // Combines the per-CTA partials in a fixed order (one CTA of 256 threads).
 __global__ void residual_final_k(const double* part, int64_t nparts, double* cheb, double* fro,
                                  int* status, double* sums = nullptr) {
@@ -397,6 +632,36 @@ static cur_status assemble_t(cur_handle* h, const cur_mat* Am, const int32_t* I,
     return CUR_OK;
 }
 
+// CUR_ERR_ARG where the workspace cannot hold W padded to whole tiles (the caller then takes
+// residual_k, which needs up to 512 r bytes less).
+template <typename TA>
+static cur_status residual_fma_t(cur_handle* h, const cur_mat* Am, const void* C, const double* U, const void* R,
+                                 int r, double* cheb, double* fro, Arena& ar, cudaStream_t st, double* sums) {
+    const int64_t m = Am->rows, n = Am->cols;
+    const int64_t ntile_n = (n + kRfB - 1) / kRfB, npad = ntile_n * kRfB, ntiles = (m + kRfB - 1) / kRfB * ntile_n;
+    float* W = ar.get<float>((size_t)r * npad);
+    const int grid = (int)std::min<int64_t>(2LL * h->num_sms, ntiles);
+    double* part = ar.get<double>((size_t)grid * 4);
+    if (!ar.ok || npad / 32 > INT_MAX) return CUR_ERR_ARG;
+    const size_t smw = (size_t)r * (kRfWK + 32) * sizeof(double);
+    CUR_TRY(smem_attr((const void*)residual_w2_k<TA>, smw));
+    residual_w2_k<TA><<<dim3((unsigned)(npad / 32), (unsigned)((r + kRfWK - 1) / kRfWK)), 256, smw, st>>>(
+        U, static_cast<const TA*>(R), r, n, npad, W);
+    CUR_CK(cudaGetLastError());
+    note_launch();
+    const size_t sm = (size_t)(2 * kRfKC + r) * kRfB * sizeof(float);
+    CUR_TRY(smem_attr((const void*)residual_fma_k<TA>, sm));
+    const int pairs = (reinterpret_cast<uintptr_t>(Am->data) % (2 * sizeof(TA))) == 0 && Am->ld % 2 == 0;
+    residual_fma_k<TA><<<grid, kRfT, sm, st>>>(static_cast<const TA*>(Am->data), m, n, Am->ld, static_cast<const TA*>(C),
+                                               W, npad, r, ntile_n, ntiles, part, pairs);
+    CUR_CK(cudaGetLastError());
+    note_launch();
+    residual_final_k<<<1, 256, 0, st>>>(part, grid, cheb, fro, h->status, sums);
+    CUR_CK(cudaGetLastError());
+    note_launch();
+    return CUR_OK;
+}
+
 template <typename TA, typename TW, int TM, int TN>
 static cur_status residual_t(cur_handle* h, const cur_mat* Am, const void* C, const double* U,
                              const void* R, int r, double* cheb, double* fro, Arena& ar,
@@ -453,6 +718,15 @@ cur_status residual_impl(cur_handle* h, const cur_mat* A, const void* C, const d
         // tensor-core (tcgen05) form where it applies; CUR_ERR_ARG means it does not
         const size_t mark = ar.off;
         const cur_status s = residual_tc_impl(h, A, C, U, R, r, cheb_out, fro_out, ar, st, sums_out);
+        if (s != CUR_ERR_ARG) return s;
+        ar.off = mark;
+        ar.ok = true;
+    }
+    if (A->dtype != CUR_F64) {
+        const size_t mark = ar.off;
+        const cur_status s = A->dtype == CUR_F32
+            ? curk::residual_fma_t<float>(h, A, C, U, R, r, cheb_out, fro_out, ar, st, sums_out)
+            : curk::residual_fma_t<__nv_bfloat16>(h, A, C, U, R, r, cheb_out, fro_out, ar, st, sums_out);
         if (s != CUR_ERR_ARG) return s;
         ar.off = mark;
         ar.ok = true;

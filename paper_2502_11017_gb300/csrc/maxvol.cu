@@ -54,7 +54,15 @@ struct MvProb {
     int32_t G;         // CTAs in its group
     int32_t rpc;       // rows per CTA
     int32_t group0;    // first slot of its group
+    int32_t kcta;      // 1: the group's first CTA holds no rows, it only keeps M^-1
+    int32_t msm;       // 1: M^-1 is kept in shared memory
 };
+// The rows of a group's CTA `part`: [lo, lo + nloc).
+__device__ __forceinline__ void part_rows(const MvProb& pr, int part, int& lo, int& nloc) {
+    const int q = part - pr.kcta;
+    lo = max(0, q) * pr.rpc;
+    nloc = q < 0 ? 0 : max(0, min(pr.p, lo + pr.rpc) - lo);
+}
 
 struct MvArgs {
     const void* basis;  // rows x r (compute type), contiguous
@@ -215,7 +223,9 @@ __global__ void __launch_bounds__(StartThreads<TB>::v, 1) mv_start(MvArgs a) {
     if (a.done[pb]) return;   // every CTA of the group leaves together: no barrier is left waiting
     const MvProb pr = a.prob[pb];
     const int r = pr.r, rs = a.r, G = pr.G;
-    const int lo = part * pr.rpc, hi = min(pr.p, lo + pr.rpc), nloc = max(0, hi - lo);
+    int lo, nloc;
+    part_rows(pr, part, lo, nloc);
+    const int hi = lo + nloc;
     const TB* basis = static_cast<const TB*>(a.basis) + pr.boff;
     TB* rows = reinterpret_cast<TB*>(smem_raw);
     const int ld = start_ld(r);
@@ -507,28 +517,36 @@ __global__ void __launch_bounds__(512) mv_lu(MvArgs a) {
 
 // ---------------------------------------------------------------- the swap iteration
 
-// The first CTA of a group keeps M^-1 (FP64) in shared memory when r <= kMsMax.
+// M^-1 is always kept in shared memory when r <= kMsMax; above, where it fits beside B.
 constexpr int kMsMax = 64;
 
 // Layout: [B slice | M^-1 (compute type) | colj | wrow] or, with the B slice in global
 // memory (a stage whose B does not fit in the shared memory of co-resident CTAs),
-// [M^-1 | colj | wrow | staging of kEngStage C rows]; while M^-1 is being refactorised,
+// [M^-1 | colj | wrow | staging of C rows]; while M^-1 is being refactorised,
 // [C(S,:) in FP64 | pivot column | pivots] over the same bytes (all dead then); after it
 // the first CTA's MinvKeeper.
-constexpr int kEngStage = 32;
-
+// A keeper CTA (MvProb::kcta) has [M^-1 as kept, and as the scratch of its refactorisation |
+// pivot column | pivots | the MinvKeeper's vectors | wrow]: it keeps a 128 x 128 double-float
+// M^-1 in shared memory (in global memory one swap's updates of it took ~30 us, the whole group
+// waiting), and the row CTAs have their shared memory to themselves.
 template <typename TB>
 struct EngineSmem {
-    __host__ __device__ static size_t head(int nloc, int r, bool gmode = false) {
-        const size_t b = gmode ? ((size_t)r * r + nloc + r + (size_t)kEngStage * r) * sizeof(TB)
-                               : ((size_t)nloc * r + (size_t)r * r + nloc + r) * sizeof(TB);
-        const size_t gj = ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int);
-        return ((b > gj ? b : gj) + 15) / 16 * 16;
+    // rows of C staged per chunk with B in global memory: eight per warp (FP32), or 32
+    static constexpr int kStage = std::is_same<TB, float>::value ? 128 : 32;
+    __host__ __device__ static size_t gj(int r) { return ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int); }
+    __host__ __device__ static size_t rows(int nloc, int r, bool gmode) {
+        return gmode ? ((size_t)r * r + nloc + r + 4 + (size_t)kStage * ((r + 3) / 4 * 4)) * sizeof(TB)
+                     : ((size_t)nloc * r + (size_t)r * r + nloc + r) * sizeof(TB);
     }
-    static size_t bytes(int nloc, int r, bool gmode = false) {
-        size_t b = head(nloc, r, gmode) + (size_t)12 * r * sizeof(double) + 64;   // keeper vectors
-        if (r <= kMsMax) b += (size_t)r * r * sizeof(double);
-        return b;
+    // offset of the MinvKeeper
+    __host__ __device__ static size_t head(int nloc, int r, bool gmode, bool kcta) {
+        const size_t b = kcta ? 0 : rows(nloc, r, gmode);
+        return ((b > gj(r) ? b : gj(r)) + 15) / 16 * 16;
+    }
+    static size_t bytes(int nloc, int r, bool gmode, bool kcta, bool msm) {
+        const size_t vec = (size_t)12 * r * sizeof(double) + 64;
+        if (kcta) return std::max(rows(nloc, r, gmode) + 16, head(0, r, gmode, true) + vec + r * sizeof(TB));
+        return head(nloc, r, gmode, false) + vec + (msm ? (size_t)r * r * sizeof(double) : 0);
     }
 };
 
@@ -543,23 +561,101 @@ __device__ __forceinline__ double coef_key_value(unsigned long long k, float) {
 }
 __device__ __forceinline__ double coef_key_value(unsigned long long k, double) { return dkey_value(k); }
 
-// Local argmax of |B| over the slice in the compute type; ties to the lowest index.
+// One pass over the B slice: with UPD, B <- B - (B(:,j) / B_ij) (B(i,:) - e_j^T) first (colj and
+// wrow = B(i,:) in shared memory); then the argmax of |B| in the compute type, ties to the
+// lowest index, and whether a NaN was met. A thread keeps one column (or four: 16-byte
+// accesses, where r and the slice's address allow), so B(i,:) - e_j is read once and its
+// indices only grow: a strict '>' keeps the lowest of equal maxima. Several rows' loads issue
+// before their arithmetic. With the slice in global memory these loads are what bounds the pass:
+// 512 threads x 4 rows x 16 bytes in flight per SM instead of 256 x 4 x 4 (one element
+// at a time where r does not divide the block). The swap iteration from a random start, M^-1 on
+// a CTA of its own: 262144 x 64 4.2 -> 1.6 ms, the polish of 262144 x 128 13.1 -> 4.3 ms.
 template <typename TB>
-__device__ __forceinline__ void engine_scan(const TB* Bs, int nloc, int r, int lo, unsigned long long& bk,
-                                            long long& bi, int& nan) {
+struct PassMax {
     TB v = (TB)-1;
-    int idx = INT_MAX;
-    int bad = 0;
-    Walk2 w(threadIdx.x, blockDim.x, r);
-    for (int e = threadIdx.x; e < nloc * r; e += blockDim.x, w.next()) {
-        const TB x = fabs(Bs[e]);
-        if (!(x <= (TB)INFINITY)) bad = 1;
-        const int id = (lo + w.i) * r + w.c;
-        if (x > v || (x == v && id < idx)) { v = x; idx = id; }
+    int idx = INT_MAX, bad = 0;
+    __device__ __forceinline__ void take(TB x, int id) {
+        const TB a = fabs(x);
+        bad |= !(a <= (TB)INFINITY);
+        if (a > v) { v = a; idx = id; }
     }
-    bk = idx == INT_MAX ? coef_key((TB)-INFINITY) : coef_key(v);
-    bi = idx == INT_MAX ? LLONG_MAX : (long long)idx;
-    nan = bad;
+};
+template <bool UPD, typename TB>
+__device__ __forceinline__ void engine_pass(TB* Bs, int nloc, int r, int lo, const TB* colj, const TB* wrow, int jstar,
+                                            unsigned long long& bk, long long& bi, int& nan) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    PassMax<TB> m;
+    bool done = false;
+    if constexpr (std::is_same<TB, float>::value) {
+        if (r % 4 == 0 && nt % (r / 4) == 0 && (reinterpret_cast<uintptr_t>(Bs) & 15) == 0) {
+            done = true;
+            const int g = r / 4, c = 4 * (tid % g), di = nt / g;
+            float w[4] = {0.f, 0.f, 0.f, 0.f};
+            if (UPD) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) w[q] = c + q == jstar ? wrow[c + q] - 1.f : wrow[c + q];
+            }
+            int i = tid / g, id = (lo + i) * r + c;
+            float* bp = Bs + (size_t)i * r + c;
+            const size_t step = (size_t)di * r;
+            auto one = [&](float4 b, float cj, float* dst, int id0) {
+                if (UPD) {
+                    b = make_float4(fmaf(-cj, w[0], b.x), fmaf(-cj, w[1], b.y), fmaf(-cj, w[2], b.z), fmaf(-cj, w[3], b.w));
+                    *reinterpret_cast<float4*>(dst) = b;
+                }
+                m.take(b.x, id0);
+                m.take(b.y, id0 + 1);
+                m.take(b.z, id0 + 2);
+                m.take(b.w, id0 + 3);
+            };
+            constexpr int U = 4;
+            for (; i + (U - 1) * di < nloc; i += U * di, id += U * di * r, bp += U * step) {
+                float4 b[U];
+                float cj[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    b[u] = *reinterpret_cast<const float4*>(bp + u * step);
+                    cj[u] = UPD ? colj[i + u * di] : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) one(b[u], cj[u], bp + u * step, id + u * di * r);
+            }
+            for (; i < nloc; i += di, id += di * r, bp += step)
+                one(*reinterpret_cast<const float4*>(bp), UPD ? colj[i] : 0.f, bp, id);
+        }
+    }
+    if (!done) {
+        const int di = nt / r;   // threads past di r have no column
+        if (tid < di * r) {
+            const int c = tid % r;
+            const TB w = UPD ? (c == jstar ? wrow[c] - (TB)1 : wrow[c]) : (TB)0;
+            int i = tid / r, id = (lo + i) * r + c;
+            TB* bp = Bs + (size_t)i * r + c;
+            const size_t step = (size_t)di * r;
+            auto one = [&](TB b, TB cj, TB* dst, int id0) {
+                if (UPD) {
+                    b = fma(-cj, w, b);
+                    *dst = b;
+                }
+                m.take(b, id0);
+            };
+            constexpr int U = 8;
+            for (; i + (U - 1) * di < nloc; i += U * di, id += U * di * r, bp += U * step) {
+                TB b[U], cj[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    b[u] = bp[u * step];
+                    cj[u] = UPD ? colj[i + u * di] : (TB)0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) one(b[u], cj[u], bp + u * step, id + u * di * r);
+            }
+            for (; i < nloc; i += di, id += di * r, bp += step) one(*bp, UPD ? colj[i] : (TB)0, bp, id);
+        }
+    }
+    bk = m.idx == INT_MAX ? coef_key((TB)-INFINITY) : coef_key(m.v);
+    bi = m.idx == INT_MAX ? LLONG_MAX : (long long)m.idx;
+    nan = m.bad;
 }
 
 // The first CTA's copy of M^-1 and its Sherman-Morrison update. For FP32/BF16 data it
@@ -571,33 +667,31 @@ struct MinvKeeper;
 
 template <>
 struct MinvKeeper<float> {
-    float* Mh;
-    float* Ml;
+    float2* Md;   // (high, low) pairs: the bytes of the FP64 entries, so a copy may be made in place
     df64* crow;   // r: C(i*,:)
     df64* brow;   // r: row i* of B
     df64* cj;     // r: column j* of M^-1, then divided by B(i*,j*)
     df64* red;    // 8 r: eighth-sums of brow
     LogAcc lacc;
-    __device__ void setup(unsigned char* base, int r, double* Mg, bool in_smem, float* gdf) {
+    // M^-1 at `own`, or after the vectors when that is null
+    __device__ void setup(unsigned char* base, int r, void* own) {
         crow = reinterpret_cast<df64*>(base);
         brow = crow + r;
         cj = brow + r;
         red = cj + r;
-        Mh = in_smem ? reinterpret_cast<float*>(red + 8 * r) : gdf;
-        Ml = Mh + r * r;
+        Md = own ? static_cast<float2*>(own) : reinterpret_cast<float2*>(red + 8 * r);
         lacc.init();
     }
     __device__ void load(const double* Mg, int r) {
         for (int e = threadIdx.x; e < r * r; e += blockDim.x) {
             const df64 v = df_from_d(Mg[e]);
-            Mh[e] = v.h;
-            Ml[e] = v.l;
+            Md[e] = make_float2(v.h, v.l);
         }
     }
     __device__ void store(double* Mg, int r) const {
-        for (int e = threadIdx.x; e < r * r; e += blockDim.x) Mg[e] = df_to_d(df64{Mh[e], Ml[e]});
+        for (int e = threadIdx.x; e < r * r; e += blockDim.x) Mg[e] = df_to_d(df64{Md[e].x, Md[e].y});
     }
-    __device__ float value(int e) const { return __fadd_rn(Mh[e], Ml[e]); }
+    __device__ float value(int e) const { return __fadd_rn(Md[e].x, Md[e].y); }
     // The update for the winner (i*, j*) with C row `ci`, in four phases that the engine
     // separates by barriers and overlaps with its own work: load the row and column j* of
     // M^-1; the partial sums of the row i* of B = C(i*,:) M^-1; that row, B(i*,j*) and the
@@ -605,7 +699,8 @@ struct MinvKeeper<float> {
     __device__ void swap_load(const float* ci, int r, int jstar) {
         for (int c = threadIdx.x; c < r; c += blockDim.x) {
             crow[c] = df64{ci[c], 0.f};
-            cj[c] = df64{Mh[c * r + jstar], Ml[c * r + jstar]};
+            const float2 m = Md[c * r + jstar];
+            cj[c] = df64{m.x, m.y};
         }
     }
     // brow = crow M^-1: eight partial sums per column, so each dependent chain is r/8 long
@@ -613,8 +708,10 @@ struct MinvKeeper<float> {
         for (int it = threadIdx.x; it < 8 * r; it += blockDim.x) {
             const int c = it % r, qt = it / r;
             df64 s{0.f, 0.f};
-            for (int k = r * qt / 8; k < r * (qt + 1) / 8; ++k)
-                s = df_add(s, df_mul_f(df64{Mh[k * r + c], Ml[k * r + c]}, crow[k].h));
+            for (int k = r * qt / 8; k < r * (qt + 1) / 8; ++k) {
+                const float2 m = Md[k * r + c];
+                s = df_add(s, df_mul_f(df64{m.x, m.y}, crow[k].h));
+            }
             red[qt * r + c] = s;
         }
     }
@@ -631,44 +728,29 @@ struct MinvKeeper<float> {
         }
         if (tid == nt - 1) lacc.mul(row_sum(r, jstar));
     }
+    __device__ static float2 sub_prod(float2 m, df64 q, df64 w) {
+        const df64 v = df_sub(df64{m.x, m.y}, df_mul(q, w));
+        return make_float2(v.h, v.l);
+    }
     // M^-1 <- M^-1 - (M^-1(:,j) / B_ij) (B(i,:) - e_j^T)
     __device__ void swap_update(int r, int jstar) {
-        const int tid = threadIdx.x, nt = blockDim.x;
-        if (nt % r == 0) {   // one column per thread, four rows at a time
-            const int c = tid % r, di = nt / r;
-            const df64 wv = c == jstar ? df_sub(brow[c], df64{1.f, 0.f}) : brow[c];
-            int i = tid / r;
-            for (; i + 3 * di < r; i += 4 * di) {
-                df64 m[4], q[4];
+        const int di = blockDim.x / r;   // a thread keeps one column, four rows at a time
+        if (threadIdx.x >= di * r) return;
+        const int c = threadIdx.x % r;
+        const df64 wv = c == jstar ? df_sub(brow[c], df64{1.f, 0.f}) : brow[c];
+        int i = threadIdx.x / r;
+        for (; i + 3 * di < r; i += 4 * di) {
+            float2 m[4];
+            df64 q[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int e = (i + u * di) * r + c;
-                    m[u] = df64{Mh[e], Ml[e]};
-                    q[u] = cj[i + u * di];
-                }
+            for (int u = 0; u < 4; ++u) {
+                m[u] = Md[(i + u * di) * r + c];
+                q[u] = cj[i + u * di];
+            }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int e = (i + u * di) * r + c;
-                    const df64 mv = df_sub(m[u], df_mul(q[u], wv));
-                    Mh[e] = mv.h;
-                    Ml[e] = mv.l;
-                }
-            }
-            for (; i < r; i += di) {
-                const int e = i * r + c;
-                const df64 mv = df_sub(df64{Mh[e], Ml[e]}, df_mul(cj[i], wv));
-                Mh[e] = mv.h;
-                Ml[e] = mv.l;
-            }
-        } else {
-            Walk2 w(tid, nt, r);
-            for (int e = tid; e < r * r; e += nt, w.next()) {
-                const df64 wv = w.c == jstar ? df_sub(brow[w.c], df64{1.f, 0.f}) : brow[w.c];
-                const df64 mv = df_sub(df64{Mh[e], Ml[e]}, df_mul(cj[w.i], wv));
-                Mh[e] = mv.h;
-                Ml[e] = mv.l;
-            }
+            for (int u = 0; u < 4; ++u) Md[(i + u * di) * r + c] = sub_prod(m[u], q[u], wv);
         }
+        for (; i < r; i += di) Md[i * r + c] = sub_prod(Md[i * r + c], cj[i], wv);
     }
     __device__ double dlog() const { return lacc.log_value(); }
 };
@@ -681,12 +763,12 @@ struct MinvKeeper<double> {
     double* cj;
     double* red;
     LogAcc lacc;
-    __device__ void setup(unsigned char* base, int r, double* Mg, bool in_smem, float*) {
+    __device__ void setup(unsigned char* base, int r, void* own) {
         crow = reinterpret_cast<double*>(base);
         brow = crow + r;
         cj = brow + r;
         red = cj + r;
-        M = in_smem ? red + 8 * r : Mg;
+        M = own ? static_cast<double*>(own) : red + 8 * r;
         lacc.init();
     }
     __device__ void load(const double* Mg, int r) {
@@ -795,22 +877,29 @@ __device__ double engine_kappa(const MinvKeeper<TB>& keep, const TB* basis, cons
     return kap;
 }
 
-// Refresh of an FP32 B slice: B = C M^-1 for nloc rows (r = 32 or 64), the
-// product of the engine's cycles after the first. C rows pass through shared memory
-// (coalesced loads) in chunks of 8 rows per warp, staged in the chunk's own rows of B; each
-// thread forms an 8 x (r/32) register tile (rows warp-uniform, columns lane + 32 j) with the
-// C values read four k at a time as one broadcast 16-byte load, so a warp issues 8 + 4 r/32
-// shared loads per 32 r/32 FMAs instead of two loads per FMA. Each entry is still one FMA
-// chain over k in order, as a dot product.
-template <int TN>
-__device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const float* Cs, int nloc, int r) {
+// Refresh of an FP32 B slice: B = C M^-1 for nloc rows, the product of the engine's cycles
+// after the first. C rows pass through shared memory (coalesced loads) in chunks of 8 rows per
+// warp; with B in shared memory (r % 4 == 0) the chunk's own rows of B hold them, with B in
+// global memory (any r) a staging area with rows of rp = 4 ceil(r / 4) words. Each thread
+// forms an 8 x TN register tile (rows warp-uniform, columns lane + 32 j, TN = ceil(r / 32))
+// with the C values read four k at a time as one broadcast 16-byte load, so a warp issues
+// 8 + 4 TN shared loads per 32 TN FMAs instead of two loads per FMA. Each entry is still one
+// FMA chain over k in order, as a dot product.
+template <int TN, bool GLOB>
+__device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const float* Cs, int nloc, int r, float* area) {
     constexpr int TM = 8;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    const int chunk = TM * nw;
+    const int chunk = TM * nw, rp = GLOB ? (r + 3) / 4 * 4 : r;
     for (int i0 = 0; i0 < nloc; i0 += chunk) {
         const int nr = min(chunk, nloc - i0);
-        float* stage = Bs + (size_t)i0 * r;
-        for (int e = tid; e < nr * r; e += nt) stage[e] = Cs[(int64_t)i0 * r + e];
+        float* stage = GLOB ? area : Bs + (size_t)i0 * r;
+        const float* src = Cs + (int64_t)i0 * r;
+        if (rp == r) {
+            for (int e = tid; e < nr * r; e += nt) stage[e] = src[e];
+        } else {
+            Walk2 w(tid, nt, r);
+            for (int e = tid; e < nr * r; e += nt, w.next()) stage[w.i * rp + w.c] = src[e];
+        }
         __syncthreads();
         float acc[TM][TN];
 #pragma unroll
@@ -819,8 +908,12 @@ __device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const 
             for (int j = 0; j < TN; ++j) acc[q][j] = 0.f;
         const float* crow[TM];
 #pragma unroll
-        for (int q = 0; q < TM; ++q) crow[q] = stage + (size_t)min(warp * TM + q, nr - 1) * r;   // rows past nr: not stored
-        for (int k = 0; k < r; k += 4) {
+        for (int q = 0; q < TM; ++q) crow[q] = stage + (size_t)min(warp * TM + q, nr - 1) * rp;   // rows past nr: not stored
+        const float* mcol[TN];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) mcol[j] = Mi + min(lane + 32 * j, r - 1);   // columns past r: not stored
+        int k = 0;
+        for (; k + 4 <= r; k += 4) {
             float4 cv[TM];
 #pragma unroll
             for (int q = 0; q < TM; ++q) cv[q] = *reinterpret_cast<const float4*>(crow[q] + k);
@@ -828,7 +921,7 @@ __device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const 
             for (int kk = 0; kk < 4; ++kk) {
                 float mv[TN];
 #pragma unroll
-                for (int j = 0; j < TN; ++j) mv[j] = Mi[(k + kk) * r + lane + 32 * j];
+                for (int j = 0; j < TN; ++j) mv[j] = mcol[j][(k + kk) * r];
 #pragma unroll
                 for (int q = 0; q < TM; ++q) {
                     const float c = kk == 0 ? cv[q].x : kk == 1 ? cv[q].y : kk == 2 ? cv[q].z : cv[q].w;
@@ -837,21 +930,37 @@ __device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const 
                 }
             }
         }
+        if (GLOB)
+            for (; k < r; ++k)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) {
+                    const float mv = mcol[j][k * r];
+#pragma unroll
+                    for (int q = 0; q < TM; ++q) acc[q][j] = fmaf(crow[q][k], mv, acc[q][j]);
+                }
         __syncthreads();
+        float* dst = Bs + (size_t)i0 * r;
 #pragma unroll
         for (int q = 0; q < TM; ++q) {
             const int i = warp * TM + q;
             if (i < nr)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) stage[(size_t)i * r + lane + 32 * j] = acc[q][j];
+                for (int j = 0; j < TN; ++j)
+                    if (lane + 32 * j < r) dst[(size_t)i * r + lane + 32 * j] = acc[q][j];
         }
-        __syncthreads();
+        if (!GLOB) __syncthreads();
     }
+    if (GLOB) __syncthreads();
 }
 
-__device__ __forceinline__ void engine_refresh_tiled(float* Bs, const float* Mi, const float* Cs, int nloc, int r) {
-    if (r == 32) refresh_tiled_tn<1>(Bs, Mi, Cs, nloc, r);
-    else refresh_tiled_tn<2>(Bs, Mi, Cs, nloc, r);
+template <bool GLOB>
+__device__ __forceinline__ void engine_refresh_tiled(float* Bs, const float* Mi, const float* Cs, int nloc, int r, float* area) {
+    switch ((r + 31) / 32) {
+        case 1: refresh_tiled_tn<1, GLOB>(Bs, Mi, Cs, nloc, r, area); break;
+        case 2: refresh_tiled_tn<2, GLOB>(Bs, Mi, Cs, nloc, r, area); break;
+        case 3: refresh_tiled_tn<3, GLOB>(Bs, Mi, Cs, nloc, r, area); break;
+        default: refresh_tiled_tn<4, GLOB>(Bs, Mi, Cs, nloc, r, area);
+    }
 }
 
 // Problems that one CTA holds alone run with kSoloThreads threads (their swaps never wait on
@@ -867,15 +976,17 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
     const MvProb pr = a.prob[pb];
     const int r = pr.r, rs = a.r, G = pr.G, tid = threadIdx.x, nt = blockDim.x;
     const bool solo = G == 1;                   // one CTA: no inter-CTA exchange at all
-    const int lo = part * pr.rpc, hi = min(pr.p, lo + pr.rpc), nloc = max(0, hi - lo);
+    int lo, nloc;
+    part_rows(pr, part, lo, nloc);
     const bool gmode = a.bglob != nullptr && pr.gmode;
+    const bool keeper = pr.kcta && part == 0;   // this CTA has no rows
+    const size_t off = EngineSmem<TB>::head(nloc, r, gmode, keeper);
     TB* Bs = gmode ? static_cast<TB*>(a.bglob) + pr.boff + (int64_t)lo * r   // nloc x r slice of B
                    : reinterpret_cast<TB*>(smem_raw);
     TB* Mi = gmode ? reinterpret_cast<TB*>(smem_raw) : Bs + (size_t)nloc * r;   // r x r: M^-1 (compute type)
     TB* colj = Mi + (size_t)r * r;              // nloc
-    TB* wrow = colj + nloc;                     // r: winning row of B, then B(i,:) - e_j
-    TB* cstage = wrow + r;                      // global-memory mode: kEngStage C rows
-    const size_t off = EngineSmem<TB>::head(nloc, r, gmode);
+    TB* wrow = keeper ? reinterpret_cast<TB*>(smem_raw + off + (size_t)12 * r * sizeof(double)) : colj + nloc;   // r: winning row of B
+    TB* cstage = reinterpret_cast<TB*>((reinterpret_cast<uintptr_t>(wrow + r) + 15) & ~(uintptr_t)15);   // global B: staged C rows
     double* Mg = a.minv64 + (int64_t)pb * minv_stride(rs);      // M^-1 in global memory (FP64)
     __shared__ long long s_w;
     __shared__ int s_nan, s_go;
@@ -888,7 +999,10 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
     const int myslot = pr.group0 + part;
     if (part == 0) {
         if (tid == 0)
-            keep.setup(smem_raw + off, r, Mg, r <= kMsMax, a.mdf ? a.mdf + (int64_t)pb * 2 * rs * rs : nullptr);
+            keep.setup(smem_raw + off, r, keeper ? static_cast<void*>(smem_raw)
+                                          : pr.msm ? nullptr
+                                          : std::is_same<TB, double>::value ? static_cast<void*>(Mg)
+                                                                            : static_cast<void*>(a.mdf + (int64_t)pb * 2 * rs * rs));
         __syncthreads();
         keep.load(Mg, r);
         for (int k = tid; k < r; k += nt) S0[k] = a.S[(int64_t)pb * rs + k];
@@ -992,28 +1106,37 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
     while (true) {
         // refresh: B slice = C slice M^-1
         __syncthreads();
-        if (part == 0) {
+        if (keeper) {
+        } else if (part == 0) {
             for (int e = tid; e < r * r; e += nt) Mi[e] = (TB)keep.value(e);
         } else {
             for (int e = tid; e < r * r; e += nt) Mi[e] = (TB)Mg[e];
         }
         __syncthreads();
-        bool tiled = false;
-        if constexpr (std::is_same<TB, float>::value) {
-            tiled = !(a.bpre && first_cycle) && !gmode && (r == 32 || r == 64);
-            if (tiled) engine_refresh_tiled(Bs, Mi, basis + (int64_t)lo * r, nloc, r);
-        }
-        if (tiled) {
-        } else if (a.bpre && first_cycle) {
+        const TB* Cs = basis + (int64_t)lo * r;
+        bool tiled = nloc == 0;
+        if (!tiled && a.bpre && first_cycle) {
             // the first cycle's B slice was formed on the tensor cores from the same M^-1
+            // (in place when the whole stage keeps its B in global memory)
+            tiled = true;
             const TB* src = static_cast<const TB*>(a.bpre) + pr.boff + (int64_t)lo * r;
-            for (int e = tid; e < nloc * r; e += nt) Bs[e] = src[e];
-        } else {
+            if (src != Bs)
+                for (int e = tid; e < nloc * r; e += nt) Bs[e] = src[e];
+        }
+        if constexpr (std::is_same<TB, float>::value) {
+            if (!tiled && gmode) {
+                engine_refresh_tiled<true>(Bs, Mi, Cs, nloc, r, cstage);
+                tiled = true;
+            } else if (!tiled && r % 4 == 0 && r >= 32) {
+                engine_refresh_tiled<false>(Bs, Mi, Cs, nloc, r, nullptr);
+                tiled = true;
+            }
+        }
+        if (!tiled) {
             // C rows pass through shared memory a chunk at a time (coalesced loads), then
             // B rows = C rows M^-1 with 8 outputs per thread in registers; the chunk's
             // own rows of Bs serve as the staging area (a separate one when B is global).
-            const TB* Cs = basis + (int64_t)lo * r;
-            const int chunk = max(1, min(kEngStage, 8 * nt / r));
+            const int chunk = max(1, min(32, 8 * nt / r));
             for (int i0 = 0; i0 < nloc; i0 += chunk) {
                 const int nr = min(chunk, nloc - i0);
                 TB* stage = gmode ? cstage : Bs + (size_t)i0 * r;
@@ -1043,7 +1166,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
         }
         first_cycle = false;
         __syncthreads();
-        engine_scan(Bs, nloc, r, lo, bk, bi, nan);
+        engine_pass<false>(Bs, nloc, r, lo, static_cast<const TB*>(nullptr), static_cast<const TB*>(nullptr), 0, bk, bi, nan);
         if (!reduce_decide()) { fin = 3; fstat = CUR_ERR_TIMEOUT; break; }
         int made = 0;
         while (true) {
@@ -1052,7 +1175,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
             if (s_go < 0) { fin = 3; fstat = CUR_ERR_NOCONV; break; }
             const long long wi = s_w;
             const int istar = (int)(wi / r), jstar = (int)(wi - (long long)istar * r);
-            const int owner = istar / pr.rpc;
+            const int owner = istar / pr.rpc + pr.kcta;
             const TB* wsrc = solo ? Bs + (size_t)(istar - lo) * r
                                   : pub + ((int64_t)(pr.group0 + owner) * 2 + par) * rs;
             // the winner's row of B; the first CTA's update of M^-1 runs in four phases
@@ -1064,7 +1187,14 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
             }
             __syncthreads();
             const TB b = wrow[jstar];
-            for (int i = tid; i < nloc; i += nt) colj[i] = Bs[i * r + jstar] / b;
+            for (int i = tid; i < nloc; i += 4 * nt) {   // four loads in flight (B may be in global memory)
+                TB x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = i + u * nt < nloc ? Bs[(size_t)(i + u * nt) * r + jstar] : (TB)0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (i + u * nt < nloc) colj[i + u * nt] = x[u] / b;
+            }
             if (part == 0) keep.swap_partials(r);
             __syncthreads();
             if (part == 0) keep.swap_finish_row(r, jstar);
@@ -1073,56 +1203,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
             ++total;
             if (part == 0) keep.swap_update(r, jstar);
             // B <- B - (B(:,j) / B_ij) (B(i,:) - e_j^T), fused with the next local argmax
-            {
-                TB v = (TB)-1;
-                int idx = INT_MAX, bad = 0;
-                if (nt % r == 0) {
-                    // each thread keeps one column (r divides the block): B(i,:) - e_j is read
-                    // once, and its ids only grow, so the first maximum is the lowest id
-                    const int c = tid % r, di = nt / r;
-                    const TB wc = c == jstar ? wrow[c] - (TB)1 : wrow[c];
-                    int i = tid / r, id = (lo + i) * r + c;
-                    TB* bp = Bs + (size_t)i * r + c;
-                    const size_t step = (size_t)di * r;
-                    // four rows at a time: their loads issue before the arithmetic
-                    for (; i + 3 * di < nloc; i += 4 * di, id += 4 * di * r, bp += 4 * step) {
-                        const TB c0 = colj[i], c1 = colj[i + di], c2 = colj[i + 2 * di], c3 = colj[i + 3 * di];
-                        const TB b0 = bp[0], b1 = bp[step], b2 = bp[2 * step], b3 = bp[3 * step];
-                        const TB x0 = fma(-c0, wc, b0), x1 = fma(-c1, wc, b1), x2 = fma(-c2, wc, b2), x3 = fma(-c3, wc, b3);
-                        bp[0] = x0;
-                        bp[step] = x1;
-                        bp[2 * step] = x2;
-                        bp[3 * step] = x3;
-                        const TB a0 = fabs(x0), a1 = fabs(x1), a2 = fabs(x2), a3 = fabs(x3);
-                        bad |= !(a0 <= (TB)INFINITY) | !(a1 <= (TB)INFINITY) | !(a2 <= (TB)INFINITY) | !(a3 <= (TB)INFINITY);
-                        if (a0 > v) { v = a0; idx = id; }
-                        if (a1 > v) { v = a1; idx = id + di * r; }
-                        if (a2 > v) { v = a2; idx = id + 2 * di * r; }
-                        if (a3 > v) { v = a3; idx = id + 3 * di * r; }
-                    }
-                    for (; i < nloc; i += di, id += di * r, bp += step) {
-                        const TB x = fma(-colj[i], wc, *bp);
-                        *bp = x;
-                        const TB ax = fabs(x);
-                        bad |= !(ax <= (TB)INFINITY);
-                        if (ax > v) { v = ax; idx = id; }
-                    }
-                } else {
-                    Walk2 w(tid, nt, r);
-                    for (int e = tid; e < nloc * r; e += nt, w.next()) {
-                        const TB wc = w.c == jstar ? wrow[w.c] - (TB)1 : wrow[w.c];
-                        const TB x = fma(-colj[w.i], wc, Bs[e]);
-                        Bs[e] = x;
-                        const TB ax = fabs(x);
-                        if (!(ax <= (TB)INFINITY)) bad = 1;
-                        const int id = (lo + w.i) * r + w.c;
-                        if (ax > v || (ax == v && id < idx)) { v = ax; idx = id; }
-                    }
-                }
-                bk = idx == INT_MAX ? coef_key((TB)-INFINITY) : coef_key(v);
-                bi = idx == INT_MAX ? LLONG_MAX : (long long)idx;
-                nan = bad;
-            }
+            engine_pass<true>(Bs, nloc, r, lo, colj, wrow, jstar, bk, bi, nan);
             par ^= 1;
             if (!reduce_decide()) { fin = 3; fstat = CUR_ERR_TIMEOUT; break; }
             if (made == r) { fin = 2; break; }
@@ -1314,15 +1395,19 @@ __global__ void pad_indices_k(int32_t* idx, const int32_t* count, int r, int64_t
 
 // ---------------------------------------------------------------- host side
 
-static const size_t kSmemBudget = 200 * 1024;
+// Shared memory planned for a CTA's rows (of 227 KB, with ~4 KB of static arrays). Up to kMsMax
+// 200 KB: a larger slice would leave problems on one CTA that are faster spread (FP64,
+// 1500 x 16 on 24 CTAs). Above, M^-1 and the start's projector leave little room.
+static size_t smem_budget(int r) { return (size_t)(r > kMsMax ? 220 : 200) * 1024; }
 static const int kSpreadRows = 64;   // fewest rows per CTA of a spread group
 
 template <typename TB>
-static int rows_cap(int r) {
+static int rows_cap(int r, bool starts, bool kcta) {
     int lo = 1, hi = 1 << 20;
     while (lo < hi) {
         const int mid = (lo + hi + 1) / 2;
-        if (EngineSmem<TB>::bytes(mid, r) <= kSmemBudget && StartSmem<TB>::bytes(mid, r) <= kSmemBudget) lo = mid;
+        if ((kcta ? EngineSmem<TB>::bytes(mid, r, false, true, false) : EngineSmem<TB>::bytes(mid, r, false, false, r <= kMsMax)) <= smem_budget(r) &&
+            (!starts || StartSmem<TB>::bytes(mid, r) <= smem_budget(r))) lo = mid;
         else hi = mid - 1;
     }
     return lo;
@@ -1476,6 +1561,7 @@ struct Stage {
     int coop_slots = 0;         // slots [0, coop_slots) hold groups of several CTAs
     bool keep_singular_set = false;
     TB* bglob = nullptr;        // B in global memory when it cannot live in shared memory
+    bool all_global = false;    // every problem's B does
     // the first cycle's B on the tensor cores (FP32, r = 32 or 64, large stages)
     float* bpre = nullptr;
     float* wh = nullptr;
@@ -1487,13 +1573,14 @@ struct Stage {
 
 template <typename TB>
 // starts: the stage runs the Algorithm 3 start (mv_start), which keeps each CTA's rows in
-// shared memory, so its problems never take the global-memory form.
-static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bool starts = false) {
+// shared memory, so its problems never take the global-memory form. may_start: a merge level,
+// whose last attempt does.
+static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bool starts = false, bool may_start = false) {
     const int P = (int)sg.probs.size();
     sg.P = P;
     int capr[129] = {0};   // rows per CTA with B in shared memory, by rank
     auto cap_of = [&](int rr) {
-        if (!capr[rr]) capr[rr] = rows_cap<TB>(rr);
+        if (!capr[rr]) capr[rr] = rows_cap<TB>(rr, starts || may_start || rr <= kMsMax, rr > kMsMax);
         return capr[rr];
     };
     int64_t tot_p = 0;
@@ -1504,11 +1591,12 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
     const bool many = P >= 2 * h->num_sms;
     int64_t elems_end = 0;
     bool anyg = false;
+    sg.all_global = true;
     for (auto& pr : sg.probs) {
         const int cap = cap_of(pr.r);
         int64_t G = (pr.p + cap - 1) / cap;
         pr.gmode = 0;
-        if (G > 1 && (many || G > h->num_sms) && !starts) pr.gmode = 1;
+        if (G > 1 && (many || G > h->num_sms - (pr.r > kMsMax)) && !starts) pr.gmode = 1;
         if (pr.gmode && many) {
             G = 1;
         } else if (G > 1 || pr.gmode) {
@@ -1519,12 +1607,23 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
             G = std::min<int64_t>(G, h->num_sms);
         }
         G = std::max<int64_t>(1, G);
+        // M^-1 has a CTA of its own where it fits no row CTA's shared memory, and where a pass
+        // over the group's B in global memory would otherwise wait for the CTA that also
+        // updates it
+        pr.msm = pr.r <= kMsMax || EngineSmem<TB>::bytes((int)((pr.p + G - 1) / G), pr.r, pr.gmode != 0, false, true) <= smem_budget(pr.r);
+        pr.kcta = (!pr.msm && !(pr.gmode && many)) || (pr.gmode && G >= 8);
+        if (!pr.gmode && (pr.p + cap - 1) / cap > h->num_sms - 1) pr.kcta = 0;   // no SM left for it
+        if (pr.kcta) {
+            G = std::min<int64_t>(G, h->num_sms - 1);
+            pr.msm = 1;
+        }
         const int rpc = (int)((pr.p + G - 1) / G);
-        G = (pr.p + rpc - 1) / rpc;
+        G = (pr.p + rpc - 1) / rpc + pr.kcta;
         pr.G = (int)G;
         pr.rpc = rpc;
         sg.max_rpc = std::max(sg.max_rpc, rpc);
         anyg |= pr.gmode != 0;
+        sg.all_global = sg.all_global && pr.gmode != 0;
         elems_end = std::max<int64_t>(elems_end, pr.boff + (int64_t)pr.p * pr.r);
     }
     int slots = 0;
@@ -1567,7 +1666,7 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
                 sg.tiles.push_back(CoefTile{pb, (int32_t)std::min<int64_t>(128, sg.probs[pb].p - i),
                                             sg.probs[pb].boff / r + i});
         const size_t mark = ar.off;
-        sg.bpre = ar.get<float>((size_t)sg.rows_total * r);
+        sg.bpre = sg.all_global ? reinterpret_cast<float*>(sg.bglob) : ar.get<float>((size_t)sg.rows_total * r);
         sg.wh = ar.get<float>((size_t)P * r * r);
         sg.wl = ar.get<float>((size_t)P * r * r);
         sg.dtiles = ar.get<CoefTile>(sg.tiles.size());
@@ -1665,15 +1764,17 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
 
     // shared memory of a launch: the largest any of its problems needs
     size_t sm_eng = 0, sm_start = 0;
+    bool wide = false;   // groups with more threads: M^-1 above kMsMax or B in global memory
     for (const auto& pr : sg.probs) {
-        sm_eng = std::max(sm_eng, EngineSmem<TB>::bytes(pr.rpc, pr.r, pr.gmode != 0));
+        sm_eng = std::max(sm_eng, EngineSmem<TB>::bytes(pr.rpc, pr.r, pr.gmode != 0, pr.kcta != 0, pr.msm != 0));
+        wide |= pr.gmode != 0 || pr.kcta != 0;
         sm_start = std::max(sm_start, StartSmem<TB>::bytes(pr.rpc, pr.r));
     }
-    const size_t sm_lu = ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int) + 64;
     CUR_TRY(set_smem_attr(mv_engine<TB>, sm_eng));
+    const size_t sm_lu = ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int) + 64;
     CUR_TRY(set_smem_attr(mv_lu<TB>, sm_lu));
     int occ_eng = 0, occ_start = 1;
-    CUR_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_eng, mv_engine<TB>, 256, sm_eng));
+    CUR_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_eng, mv_engine<TB>, wide ? kSoloThreads : 256, sm_eng));
     if (aca_start) {
         CUR_TRY(set_smem_attr(mv_start<TB>, sm_start));
         CUR_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_start, mv_start<TB>, StartThreads<TB>::v, sm_start));
@@ -1734,7 +1835,7 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
         MvArgs aw = a;
         aw.cta_base = w.first;
         void* args[] = {&aw};
-        CUR_TRY(launch_coop((const void*)mv_engine<TB>, dim3(w.second), dim3(256), args, sm_eng, st));
+        CUR_TRY(launch_coop((const void*)mv_engine<TB>, dim3(w.second), dim3(wide ? kSoloThreads : 256), args, sm_eng, st));
         note_launch();
     }
     return CUR_OK;
@@ -1923,7 +2024,7 @@ static cur_status merge_level_t(cur_handle* h, const TB* basis, int64_t p, int r
         pr.p = 2 * r;
         lv.probs.push_back(pr);
     }
-    CUR_TRY(stage_setup<TB>(h, r, lv, ar));
+    CUR_TRY(stage_setup<TB>(h, r, lv, ar, false, true));
     CUR_TRY(stage_tables(lv, st));
     CUR_TRY(stage_init(lv, idle, st));
     mv_iota<<<nblk(npairs * r), 256, 0, st>>>(lv.S, npairs, r, 0);
@@ -2771,7 +2872,7 @@ static cur_status bat_rows(cur_handle* h, const float* basis, const std::vector<
             pr.gid_arr = cand + (int64_t)q * 2 * rs;
             lv.probs.push_back(pr);
         }
-        CUR_TRY(stage_setup<float>(h, rs, lv, ar));
+        CUR_TRY(stage_setup<float>(h, rs, lv, ar, false, true));
         CUR_TRY(stage_tables(lv, st));
         CUR_TRY(stage_init(lv, nullptr, st));
         bat_iota_k<<<nblk((int64_t)Q * rs), 256, 0, st>>>(rr, nullptr, Q, rs, 0, lv.S);

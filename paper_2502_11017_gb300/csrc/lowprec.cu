@@ -29,6 +29,7 @@
 #include <climits>
 
 #include "common.cuh"
+#include "gj.cuh"
 #include "internal.h"
 #include "tc.cuh"
 
@@ -133,51 +134,71 @@ __device__ __forceinline__ void lp_requant(const float* M, int pitch, int r, int
     __syncthreads();
 }
 
-// The start of the phase, on the device (one CTA): S = S0; nothing more when `idle` is set;
+// The start of the phase, on the device (one cluster): S = S0; nothing more when `idle` is set;
 // the given FP64 inverse of C(S0,:) when it is valid (minv_flag NULL, CUR_OK or
 // CUR_ERR_NOCONV); else C(S0,:) in FP64, its inverse and log|det| (a singular start ends the
 // phase with CUR_ERR_SINGULAR). M^-1 is kept as hi + lo floats; W = (M^-1)^T rounded. Also
 // clears the loop's grid-barrier counter.
-template <bool F8>
-__global__ void lp_setup_k(const float* __restrict__ C, int r, int ldk, const int32_t* S0, int32_t* S,
+template <bool F8, int RU, int CPW>
+__global__ void __launch_bounds__(32 * kGjWarps) lp_setup_k(const float* __restrict__ C, int r, int ldk, const int32_t* S0, int32_t* S,
                            const double* minv_in, const int* minv_flag, const int* idle, void* W, float* winv,
                            float* Mh, float* Ml, LpCtl* ctl, unsigned* gbar) {
-    extern __shared__ double lsm[];
-    double* M = lsm;                   // r x r
-    double* colk = M + r * r;          // r
-    int* piv = reinterpret_cast<int*>(colk + r);
-    const int tid = threadIdx.x;
-    for (int k = tid; k < r; k += blockDim.x) S[k] = S0[k];
-    if (tid == 0) {
-        *gbar = 0u;
-        ctl->status = CUR_OK;
-        ctl->done = 0;
-        ctl->swaps = 0;
-        ctl->logvol = 0.0;
+    extern __shared__ __align__(16) unsigned char lsm[];
+    const GjSmem gs(lsm, r);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const unsigned rank = gj_rank();
+    if (rank == 0) {
+        for (int k = tid; k < r; k += blockDim.x) S[k] = S0[k];
+        if (tid == 0) {
+            *gbar = 0u;
+            ctl->status = CUR_OK;
+            ctl->done = 0;
+            ctl->swaps = 0;
+            ctl->logvol = 0.0;
+        }
     }
     if (idle && *idle) {
-        if (tid == 0) ctl->done = 1;
+        if (rank == 0 && tid == 0) ctl->done = 1;
         return;
     }
     const bool given = minv_in && (!minv_flag || *minv_flag == CUR_OK || *minv_flag == CUR_ERR_NOCONV);
     if (given) {
+        if (rank != 0) return;
         for (int e = tid; e < r * r; e += blockDim.x) split_d(minv_in[e], Mh[e], Ml[e]);
     } else {
         double mx = 0.0;
-        for (int e = tid; e < r * r; e += blockDim.x) {
-            const double x = (double)C[(int64_t)S0[e / r] * r + (e % r)];
-            M[e] = x;
-            mx = fmax(mx, fabs(x));
-        }
+        for (int e = tid; e < r * r; e += blockDim.x) mx = fmax(mx, fabs((double)C[(int64_t)S0[e / r] * r + (e % r)]));
         mx = block_max(mx);
+        int c0, n;
+        gj_columns(r, CPW, c0, n);
+        double v[CPW][RU];
+#pragma unroll
+        for (int q = 0; q < CPW; ++q)
+#pragma unroll
+            for (int u = 0; u < RU; ++u) {
+                const int i = lane + 32 * u;
+                v[q][u] = q < n && i < r ? (double)C[(int64_t)S0[i] * r + c0 + q] : 0.0;
+            }
         double lv = 0.0;
-        const int sing = gj_inverse(M, r, colk, piv, (double)r * 2.220446049250313e-16 * mx, &lv);
-        if (sing) {
-            if (tid == 0) { ctl->status = CUR_ERR_SINGULAR; ctl->done = 1; ctl->logvol = -INFINITY; }
+        const int res = gj_flow<RU, CPW>(gs, r, (double)r * 2.220446049250313e-16 * mx, v, c0, n, &lv);
+        if (res) {
+            if (rank == 0 && tid == 0) { ctl->status = res == 2 ? CUR_ERR_TIMEOUT : CUR_ERR_SINGULAR; ctl->done = 1; ctl->logvol = -INFINITY; }
             return;
         }
-        for (int e = tid; e < r * r; e += blockDim.x) split_d(M[e], Mh[e], Ml[e]);
-        if (tid == 0) ctl->logvol = lv;
+#pragma unroll
+        for (int q = 0; q < CPW; ++q)
+            if (q < n) {
+                const int c = gs.perm[c0 + q];
+#pragma unroll
+                for (int u = 0; u < RU; ++u) {
+                    const int i = lane + 32 * u;
+                    if (i < r) split_d(v[q][u], Mh[i * r + c], Ml[i * r + c]);
+                }
+            }
+        if (rank == 0 && tid == 0) ctl->logvol = lv;
+        __threadfence();
+        gj_cluster_sync();   // the other CTAs' columns of Mh
+        if (rank != 0) return;
     }
     __syncthreads();
     lp_requant<F8>(Mh, r, r, ldk, W, winv);
@@ -742,10 +763,12 @@ static cur_status lowprec_phase_t(cur_handle* h, const float* C, int64_t p, int 
     else
         lp_quant_c<<<qgrid, 256, 0, st>>>(C, p, r, ldk, static_cast<__nv_bfloat16*>(Cq));
     CUR_CK(cudaGetLastError());
-    const size_t sm_setup = (size_t)r * r * sizeof(double) + (size_t)r * sizeof(double) + (size_t)r * sizeof(int) + 64;
-    CUR_TRY(smem_attr((const void*)lp_setup_k<F8>, sm_setup));
-    lp_setup_k<F8><<<1, 256, sm_setup, st>>>(C, r, ldk, S0, S, minv_in, minv_flag, idle, W, winv, Mh, Ml, ctl, gbar);
-    CUR_CK(cudaGetLastError());
+    int nc, cpw;
+    gj_plan(r, 1, h->num_sms, &nc, &cpw);
+#define LP_SETUP(RU, CPW) lp_setup_k<F8, RU, CPW>
+    CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, LP_SETUP), nc, nc, GjSmem::bytes(r), st, C, r, ldk, S0, S, minv_in, minv_flag,
+                      idle, W, winv, Mh, Ml, ctl, gbar));
+#undef LP_SETUP
     LpLoop la{};
     la.p = p;
     la.r = r;

@@ -12,8 +12,8 @@
 // each handled by one CTA or by a group of co-resident CTAs:
 //   mv_start  : Algorithm 3 (axis 0) on the problem's rows -> start set S
 //               (implicit Gram-Schmidt, one group barrier per pick)
-//   mv_lu     : one CTA per problem, FP64 Gauss-Jordan inverse of C(S,:) with
-//               partial pivoting, log|det|
+//   mv_lu     : a CTA or a cluster of CTAs per problem, FP64 Gauss-Jordan inverse of C(S,:)
+//               with partial pivoting, log|det| (gj.cuh)
 //   mv_engine : the whole swap iteration of a stage in one launch. Each CTA keeps
 //               its slice of B in shared memory (FP32 for FP32/BF16 data, FP64 for
 //               FP64 data; in global memory for a problem too large for that), and
@@ -37,6 +37,7 @@
 
 #include "common.cuh"
 #include "df64.cuh"
+#include "gj.cuh"
 #include "internal.h"
 
 namespace curk {
@@ -455,21 +456,23 @@ __global__ void __launch_bounds__(StartThreads<TB>::v, 1) mv_start(MvArgs a) {
 
 // ---------------------------------------------------------------- FP64 inverse of C(S,:)
 
-template <typename TB>
-__global__ void __launch_bounds__(512) mv_lu(MvArgs a) {
+// One cluster per problem (gj_plan): a stage of one or a few problems spreads each inverse over
+// up to eight SMs, a stage of many keeps one CTA each. 128 x 128: 717 -> 240 us for one problem,
+// 719 -> 474 us for 16; 1436 -> 1631 us for 256 on one CTA each (FP64-bound either way).
+template <typename TB, int RU, int CPW>
+__global__ void __launch_bounds__(32 * kGjWarps) mv_lu(MvArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int pb = blockIdx.x;
-    if (threadIdx.x == 0) a.bar[pb] = 0u;   // the swap engine's group barrier starts from zero
+    const unsigned rank = gj_rank();
+    const int pb = (int)(blockIdx.x / gj_size());
+    if (rank == 0 && threadIdx.x == 0) a.bar[pb] = 0u;   // the swap engine's group barrier starts from zero
     if (a.done[pb] || !a.lu_mask[pb]) return;
     const MvProb pr = a.prob[pb];
-    const int r = pr.r, rs = a.r, tid = threadIdx.x, nt = blockDim.x;
-    double* M = reinterpret_cast<double*>(smem_raw);  // r x r, inverted in place
-    double* colk = M + r * r;
-    int* piv = reinterpret_cast<int*>(colk + r);
+    const int r = pr.r, rs = a.r, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    const GjSmem gs(smem_raw, r);
     __shared__ double s_max;
     const TB* basis = static_cast<const TB*>(a.basis) + pr.boff;
     const int32_t* S = a.S + (int64_t)pb * rs;
-    // C(S,:) in FP64; its maximum magnitude in the data's type (no FP64 comparisons)
+    // C(S,:)'s maximum magnitude in the data's type (no FP64 comparisons)
     using TS = typename std::conditional<std::is_same<TB, double>::value, double, float>::type;
     TS mx = 0;
     int bad = 0;
@@ -479,14 +482,13 @@ __global__ void __launch_bounds__(512) mv_lu(MvArgs a) {
         TS x = 0;
         if (s < 0 || s >= pr.p) bad = 1; else x = (TS)basis[(int64_t)s * r + c];
         if (!isfinite(x)) bad = 2;
-        M[e] = (double)x;
         mx = fmax(mx, fabs(x));
     }
-    bad = __syncthreads_or(bad);
+    bad = __syncthreads_or(bad == 2) ? 2 : (__syncthreads_or(bad == 1) ? 1 : 0);
     {
         __shared__ TS sm[32];
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if ((tid & 31) == 0) sm[tid >> 5] = mx;
+        if (lane == 0) sm[tid >> 5] = mx;
         __syncthreads();
         if (tid == 0) {
             TS t = 0;
@@ -496,23 +498,49 @@ __global__ void __launch_bounds__(512) mv_lu(MvArgs a) {
         __syncthreads();
     }
     if (bad) {
-        if (tid == 0) {
+        if (rank == 0 && tid == 0) {
             a.pstatus[pb] = bad == 2 ? CUR_ERR_NONFINITE : CUR_ERR_ARG;
             a.done[pb] = 1;
             set_status(a.status, bad == 2 ? CUR_ERR_NONFINITE : CUR_ERR_ARG);
         }
         return;
     }
+    int c0, n;
+    gj_columns(r, CPW, c0, n);
+    double v[CPW][RU];
+#pragma unroll
+    for (int q = 0; q < CPW; ++q)
+#pragma unroll
+        for (int u = 0; u < RU; ++u) {
+            const int i = lane + 32 * u;
+            v[q][u] = q < n && i < r ? (double)basis[(int64_t)S[i] * r + c0 + q] : 0.0;
+        }
     double lv = 0.0;
-    const int sing = gj_inverse(M, r, colk, piv, (double)r * kEps * s_max, &lv);
-    if (sing) {
-        if (tid == 0) { a.pstatus[pb] = CUR_ERR_SINGULAR; a.done[pb] = 1; a.logvol[pb] = -INFINITY; }
+    const int res = gj_flow<RU, CPW>(gs, r, (double)r * kEps * s_max, v, c0, n, &lv);
+    if (res) {
+        if (rank == 0 && tid == 0) {
+            a.pstatus[pb] = res == 2 ? CUR_ERR_TIMEOUT : CUR_ERR_SINGULAR;
+            a.done[pb] = 1;
+            a.logvol[pb] = -INFINITY;
+            if (res == 2) set_status(a.status, CUR_ERR_TIMEOUT);
+        }
         return;
     }
-    if (tid == 0) a.logvol[pb] = lv;
     double* out64 = a.minv64 + (int64_t)pb * minv_stride(rs);
-    for (int e = tid; e < r * r; e += nt) out64[e] = M[e];
-    if (tid == 0) out64[r * r] = 0.0;   // fresh: no drift
+    if (rank == 0 && tid == 0) {
+        a.logvol[pb] = lv;
+        out64[r * r] = 0.0;   // fresh: no drift
+    }
+#pragma unroll
+    for (int q = 0; q < CPW; ++q)
+        if (q < n) {
+            const int c = gs.perm[c0 + q];
+#pragma unroll
+            for (int u = 0; u < RU; ++u) {
+                const int i = lane + 32 * u;
+                if (i < r) out64[(int64_t)i * r + c] = v[q][u];
+            }
+        }
 }
 
 // ---------------------------------------------------------------- the swap iteration
@@ -1771,8 +1799,6 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
         sm_start = std::max(sm_start, StartSmem<TB>::bytes(pr.rpc, pr.r));
     }
     CUR_TRY(set_smem_attr(mv_engine<TB>, sm_eng));
-    const size_t sm_lu = ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int) + 64;
-    CUR_TRY(set_smem_attr(mv_lu<TB>, sm_lu));
     int occ_eng = 0, occ_start = 1;
     CUR_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_eng, mv_engine<TB>, wide ? kSoloThreads : 256, sm_eng));
     if (aca_start) {
@@ -1815,9 +1841,13 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
             note_launch();
         }
     }
-    mv_lu<TB><<<P, 512, sm_lu, st>>>(a);
-    CUR_CK(cudaGetLastError());
-    note_launch();
+    {
+        int nc, cpw;
+        gj_plan(r, P, h->num_sms, &nc, &cpw);
+#define MV_LU(RU, CPW) mv_lu<TB, RU, CPW>
+        CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, MV_LU), P * nc, nc, GjSmem::bytes(r), st, a));
+#undef MV_LU
+    }
     if (sg.bpre) {
         // the first cycle's B = C M^-1 of every problem on the tensor cores
         CUR_TRY(coef_tc_launch(h, reinterpret_cast<const float*>(basis), sg.rows_total, r, sg.minv64, minv_stride(r), P,

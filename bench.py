@@ -436,7 +436,7 @@ def run_ours(args):
     bytes_per_pass = m * n * 4
     avg_pass_ms = pass_ms / max(1, pass_n)
     achieved = bytes_per_pass / (avg_pass_ms / 1000.0) / 1e9 if pass_n else None
-    roof = {"bound": "hbm", "kernel": "aca_cols_pass (Algorithm 3 pass, A^T q)",
+    roof = {"bound": "hbm", "kernel": "aca_cols_ring (Algorithm 3 pass, A^T q)",
             "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / peaks["hbm_gbs"] if achieved else None,
             "peak_kind": kind, "traffic": traffic_record(),

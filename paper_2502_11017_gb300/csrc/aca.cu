@@ -86,6 +86,17 @@ __device__ __forceinline__ void acc_add(Dot2& a, float x, int mode, double, floa
     if (mode == kNorm) a.add_sq(x); else a.add(x, qh, ql);
 }
 
+// four terms, in their order
+__device__ __forceinline__ void acc_add4(DotD& a, const double* x, int mode, const double* q, const float*, const float*) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc_add(a, x[u], mode, q[u], 0.f, 0.f);
+}
+__device__ __forceinline__ void acc_add4(Dot2& a, const float* x, int mode, const double*, const float* qh, const float* ql) {
+    if (mode == kDot) { a.add4(x, qh, ql); return; }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a.add_sq(x[u]);
+}
+
 // Partial sums travel as FP64 for FP64 data and as double-float pairs otherwise.
 template <typename TA>
 using PartT = typename std::conditional<std::is_same<TA, double>::value, double, df64>::type;
@@ -112,7 +123,8 @@ __device__ __forceinline__ T warp_sum_t(T v) {
 // part[rc * n + j] = sum over rows i of chunk rc of a_ij * q_i (kDot) or a_ij^2 (kNorm).
 // grid = (ceil(n / (32 CPL)), RC), block = 256 (8 warps). Warp w takes rows r0 + w,
 // r0 + w + 8, ...; lane l takes the CPL columns 32 CPL blockIdx.x + CPL l .. (CPL = 4,
-// or 8 for BF16: 16 bytes per lane and row either way).
+// or 8 for BF16: 16 bytes per lane and row either way). For FP64, for rows that do
+// not lie on 16 bytes, and for small matrices (see ring_pays).
 template <typename TA, int MODE, bool VEC>
 __global__ void __launch_bounds__(256) aca_cols_pass(const TA* __restrict__ A, int64_t m, int64_t n,
                                                      int64_t ld, int64_t chunk,
@@ -133,56 +145,23 @@ __global__ void __launch_bounds__(256) aca_cols_pass(const TA* __restrict__ A, i
     const bool full = VEC && (col + CPL - 1 < n);
     AccOf<TA> acc[CPL];
     int64_t i = r0 + warp;
-    if constexpr (std::is_same<TA, __nv_bfloat16>::value && MODE == kDot) {
-        // BF16: about 12 FP32 operations per 2-byte element, so the sums of four rows take
-        // long enough that the next four rows' loads are issued before them (same order of
-        // summation as the loop below)
-        if (full && i + 24 < r1) {
-            uint4 xr[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) xr[u] = __ldcs(reinterpret_cast<const uint4*>(A + (i + 8 * u) * ld + col));
-            while (true) {
-                const int64_t inext = i + 32;
-                const bool more = inext + 24 < r1;
-                uint4 xn[4];
-                if (more) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        xn[u] = __ldcs(reinterpret_cast<const uint4*>(A + (inext + 8 * u) * ld + col));
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float h = qh[i + 8 * u], l = ql[i + 8 * u];
-                    const uint32_t w[4] = {xr[u].x, xr[u].y, xr[u].z, xr[u].w};
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        acc_add(acc[2 * k], __uint_as_float(w[k] << 16), MODE, 0.0, h, l);
-                        acc_add(acc[2 * k + 1], __uint_as_float(w[k] & 0xffff0000u), MODE, 0.0, h, l);
-                    }
-                }
-                i = inext;
-                if (!more) break;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) xr[u] = xn[u];
-            }
-        }
-    }
     for (; i + 24 < r1; i += 32) {
         V x[4][CPL];
+        double qd[4];
+        float h[4], l[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const TA* row = A + (i + 8 * u) * ld;
             if (full) loadc(row + col, x[u]); else loadc_guard<CPL>(row, col, n, x[u]);
+            if (MODE == kDot) {
+                if (std::is_same<TA, double>::value) qd[u] = q64[i + 8 * u];
+                else { h[u] = qh[i + 8 * u]; l[u] = ql[i + 8 * u]; }
+            }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            double qd = 0.0; float h = 0.f, l = 0.f;
-            if (MODE == kDot) {
-                if (std::is_same<TA, double>::value) qd = q64[i + 8 * u];
-                else { h = qh[i + 8 * u]; l = ql[i + 8 * u]; }
-            }
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) acc_add(acc[c], x[u][c], MODE, qd, h, l);
+        for (int c = 0; c < CPL; ++c) {
+            const V xc[4] = {x[0][c], x[1][c], x[2][c], x[3][c]};
+            acc_add4(acc[c], xc, MODE, qd, h, l);
         }
     }
     for (; i < r1; i += 8) {
@@ -212,8 +191,178 @@ __global__ void __launch_bounds__(256) aca_cols_pass(const TA* __restrict__ A, i
     }
 }
 
-// out[i] = sum_j a_ij * q_j (kDot) or a_ij^2 (kNorm); one warp per row.
-template <typename TA, int MODE, bool VEC>
+// ---- the column pass over a large matrix: A through shared memory
+//
+// The same sums (warp w takes rows r0 + w, r0 + w + 8, ... of a chunk, lane l its CPL columns),
+// each lane bringing the 16 bytes per row that it will itself sum by cp.async, kRingStages - 1
+// stages of four rows ahead: 96 KB in flight per SM with no register held for it and nothing
+// to synchronise. (Loaded DRAM answers after ~1.4 us, so 6.8 TB/s want 64 KB in flight; the
+// direct kernel's BF16 form held 32 KB in registers and waited: 1.98 ms a pass of
+// 262144 x 16384, 0.64 of the copy rate. TMA boxes of 32 rows x 512 bytes into the same ring
+// came back at 21 bytes per clock and SM however many were in flight.) BF16 has twice the
+// elements per byte, nine FMA-pipe operations each: packed pairs (Dot2x2) leave the issue slots
+// for the loads and the conversion, and the FMA pipe bounds it. At 16384 x 16384: FP32 181 ->
+// 154 us (6.95 TB/s, HBM), BF16 161 -> 115 us (4.7 TB/s). The stage's entries of q come the same way as (h, h, l, l),
+// ready pairs for one broadcast load per row. A CTA's items (a column tile of a chunk) follow
+// one another in one pipeline; neighbouring CTAs take neighbouring tiles of the same rows.
+constexpr int kRingStages = 3;
+
+// Below these a matrix stays in L2 and the direct kernel's shorter start counts (us a pass, ring and
+// direct: FP32 4096 x 4096 17.6 and 16.6, 8192 x 4096 29.7 and 31.5, 8192 x 8192 45.8 and 55.4; BF16
+// 2048 x 1024 8.6 and 8.7, 2048 x 2048 8.8 and 9.7, 4096 x 4096 16.8 and 23.2, 8192 x 8192 45.7 and
+// 84.0). FP64 stays with the direct kernel (8192 x 8192 136 and 128).
+static bool ring_pays(cur_dtype dt, int64_t m, int64_t n) {
+    if (dt == CUR_F64) return false;
+    return m * n * (int64_t)dtype_size(dt) >= (dt == CUR_BF16 ? 6LL << 20 : 96LL << 20);
+}
+template <typename TA> constexpr cur_dtype kDtypeOf = CUR_F32;
+template <> constexpr cur_dtype kDtypeOf<double> = CUR_F64;
+template <> constexpr cur_dtype kDtypeOf<__nv_bfloat16> = CUR_BF16;
+
+// One 16- or 4-byte copy; the bytes past `valid` are zeros.
+__device__ __forceinline__ void ring_copy16(uint32_t dst, const void* src, int valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst), "l"(src), "r"(valid) : "memory");
+}
+__device__ __forceinline__ void ring_copy4(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(dst), "l"(src) : "memory");
+}
+
+template <typename TA, int MODE>
+struct ColAcc {
+    static constexpr int CPL = ColsPerLane<TA>::v;
+    using Q = ulonglong2;   // (h, h), (l, l)
+    Dot2x2 acc[CPL / 2];
+    // a stage's four entries: word w of entry u comes by lane 4 u + w
+    static constexpr int kQLanes = 16;
+    __device__ __forceinline__ static int q_row(int lane) { return 8 * (lane >> 2); }
+    // rows p, p + step, ... (a stage's N, or fewer at an item's end) and their entries of q
+    template <int N>
+    __device__ __forceinline__ void add(const unsigned char* p, uint32_t step, const Q* qp) {
+        uint32_t w[N][4];
+        Q q[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            const uint4 x = *reinterpret_cast<const uint4*>(p + u * step);
+            w[u][0] = x.x; w[u][1] = x.y; w[u][2] = x.z; w[u][3] = x.w;
+            if (MODE == kDot) q[u] = qp[u];
+        }
+#pragma unroll
+        for (int k = 0; k < CPL / 2; ++k) {
+            uint64_t x[N];
+#pragma unroll
+            for (int u = 0; u < N; ++u) {
+                uint64_t a;
+                if constexpr (sizeof(TA) == 4) a = pk(__uint_as_float(w[u][2 * k]), __uint_as_float(w[u][2 * k + 1]));
+                else a = pk(__uint_as_float(w[u][k] << 16), __uint_as_float(w[u][k] & 0xffff0000u));
+                x[u] = MODE == kNorm ? acc[k].term_sq(a) : acc[k].term(a, q[u].x, q[u].y);
+            }
+            if constexpr (N == 4) acc[k].c = add2(acc[k].c, add2(add2(x[0], x[1]), add2(x[2], x[3])));
+            else acc[k].c = add2(acc[k].c, x[0]);
+        }
+    }
+    __device__ __forceinline__ df64 value(int c) const { return part_value(acc[c >> 1].half(c & 1)); }
+};
+template <typename TA, int MODE>
+__global__ void __launch_bounds__(256, 3) aca_cols_ring(const TA* __restrict__ A, int64_t m, int64_t n, int64_t ld,
+                                                        int64_t chunk, int64_t coltiles, int64_t items,
+                                                        const float* __restrict__ qh, const float* __restrict__ ql,
+                                                        df64* __restrict__ part,
+                                                        const int* __restrict__ stop) {
+    using Acc = ColAcc<TA, MODE>;
+    using Q = typename Acc::Q;
+    constexpr int CPL = Acc::CPL, TW = 32 * CPL, LB = 16;   // LB: bytes of a lane's row
+    constexpr uint32_t row_b = 32 * LB, stage_b = 8 * 4 * row_b;
+    extern __shared__ __align__(16) unsigned char ring_raw[];   // stage, warp, row, lane
+    __shared__ df64 red[8][TW];
+    __shared__ __align__(16) Q qring[kRingStages][8][4];
+    if (*stop) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned char* mine = ring_raw + (warp * 4 * 32 + lane) * LB;
+    const uint32_t mine_s = (uint32_t)__cvta_generic_to_shared(mine);
+    const uint32_t q_s = (uint32_t)__cvta_generic_to_shared(&qring[0][warp][0]) + 4 * lane;
+    const int64_t s8 = 8 * ld * (int64_t)sizeof(TA);
+    // where the next stage comes from: `left` rows of the item remain, fp is this warp's first
+    int64_t fit = blockIdx.x;
+    int left = 0, valid = 0;
+    const unsigned char* fp = nullptr;
+    const float* fq = nullptr;
+    uint32_t fdst = mine_s, fqd = q_s;
+    const uint32_t fend = mine_s + kRingStages * stage_b;
+    const bool qlane = MODE == kDot && lane < Acc::kQLanes;
+    auto copy_row = [&](uint32_t dst, const unsigned char* src) { ring_copy16(dst, src, valid); };
+    auto fetch = [&]() {
+        if (left <= 0 && fit < items) {
+            const int64_t rc = fit / coltiles, ct = fit - rc * coltiles, r0 = rc * chunk + warp, col = ct * TW + lane * CPL;
+            left = (int)min(chunk, m - rc * chunk);
+            valid = (int)max((int64_t)0, min((int64_t)LB, (n - col) * (int64_t)sizeof(TA)));
+            fp = reinterpret_cast<const unsigned char*>(A + r0 * ld + (valid ? col : 0));
+            if (MODE == kDot) fq = (lane & 2 ? ql : qh) + r0 + Acc::q_row(lane);
+            fit += gridDim.x;
+        }
+        const int own = left - warp;   // rows warp, warp + 8, ... below left
+        if (own > 24) {   // all four rows
+            const unsigned char *p1 = fp + s8, *p2 = p1 + s8, *p3 = p2 + s8;
+            copy_row(fdst, fp);
+            copy_row(fdst + row_b, p1);
+            copy_row(fdst + 2 * row_b, p2);
+            copy_row(fdst + 3 * row_b, p3);
+            if (qlane) ring_copy4(fqd, fq);
+            fp = p3 + s8;
+            if (MODE == kDot) fq += 32;
+        } else {           // an item's end
+            for (int u = 0; 8 * u < own; ++u) copy_row(fdst + u * row_b, fp + u * s8);
+            if (qlane && Acc::q_row(lane) < own) ring_copy4(fqd, fq);
+        }
+        left -= 32;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        fdst += stage_b;
+        fqd += (uint32_t)sizeof(qring[0]);
+        if (fdst == fend) { fdst = mine_s; fqd = q_s; }
+    };
+#pragma unroll
+    for (int s = 0; s < kRingStages - 1; ++s) fetch();
+    const unsigned char* src = mine;
+    const Q* q = qring[0][warp];
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+        const int64_t rc = it / coltiles, ct = it - rc * coltiles;
+        Acc acc;
+        for (int rows = (int)min(chunk, m - rc * chunk); rows > 0; rows -= 32) {
+            asm volatile("cp.async.wait_group %0;" :: "n"(kRingStages - 2) : "memory");
+            if (MODE == kDot) __syncwarp();   // the other lanes' words of q; q is read before its slot is filled again
+            fetch();
+            if (rows >= 32) {
+                acc.template add<4>(src, row_b, q);
+            } else {
+                for (int u = 0; u < 4 && warp + 8 * u < rows; ++u) acc.template add<1>(src + u * row_b, 0, q + u);
+            }
+            src += stage_b;
+            q += 8 * 4;
+            if (src == mine + kRingStages * stage_b) { src = mine; q = qring[0][warp]; }
+        }
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) red[warp][lane * CPL + k] = acc.value(k);
+        __syncthreads();
+        if (threadIdx.x < TW) {
+            const int64_t j = ct * TW + threadIdx.x;
+            if (j < n) {
+                const df64 s0 = part_add(red[0][threadIdx.x], red[1][threadIdx.x]);
+                const df64 s1 = part_add(red[2][threadIdx.x], red[3][threadIdx.x]);
+                const df64 s2 = part_add(red[4][threadIdx.x], red[5][threadIdx.x]);
+                const df64 s3 = part_add(red[6][threadIdx.x], red[7][threadIdx.x]);
+                part[rc * n + j] = part_add(part_add(s0, s1), part_add(s2, s3));
+            }
+        }
+        __syncthreads();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// out[i] = sum_j a_ij * q_j (kDot) or a_ij^2 (kNorm); one warp per kRowsPer rows (4, or 1
+// below two CTAs per SM), so that each entry of q serves that many loads of A. VEC: four consecutive columns per lane (16 bytes of
+// FP32); else lane l takes the columns l, l + 32, ...: 128-byte runs whatever the alignment (one
+// 4-byte access per row; four strided by lane, each touching every line, took 92 us a pass at
+// 20001 x 3001 FP32 (2.6 TB/s), this 61).
+template <typename TA, int MODE, bool VEC, int kRowsPer>
 __global__ void __launch_bounds__(256) aca_rows_pass(const TA* __restrict__ A, int64_t m, int64_t n,
                                                      int64_t ld, const double* __restrict__ q64,
                                                      const float* __restrict__ qh,
@@ -221,27 +370,49 @@ __global__ void __launch_bounds__(256) aca_rows_pass(const TA* __restrict__ A, i
                                                      PartT<TA>* __restrict__ out,
                                                      const int* __restrict__ stop) {
     using V = typename ValT<TA>::type;
+    constexpr bool F64 = std::is_same<TA, double>::value;
+    constexpr int W = VEC ? 4 : 1, U = VEC ? 1 : 4;   // columns per access; accesses in flight per row
     if (*stop) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < m; row += (int64_t)gridDim.x * 8) {
+    for (int64_t row = ((int64_t)blockIdx.x * 8 + warp) * kRowsPer; row < m; row += (int64_t)gridDim.x * 8 * kRowsPer) {
+        const int rows = (int)min((int64_t)kRowsPer, m - row);
         const TA* a = A + row * ld;
-        AccOf<TA> acc;
-        for (int64_t j = (int64_t)lane * 4; j < n; j += 128) {
-            V x[4];
-            if (VEC && j + 3 < n) load4(a + j, x); else load4_guard(a, j, n, x);
+        AccOf<TA> acc[kRowsPer];
+        for (int64_t j0 = (int64_t)lane * W; j0 < n; j0 += 32 * W * U) {
+            V x[kRowsPer][U][W];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int64_t jj = j + c;
-                double qd = 0.0; float h = 0.f, l = 0.f;
-                if (MODE == kDot && jj < n) {
-                    if (std::is_same<TA, double>::value) qd = q64[jj];
-                    else { h = qh[jj]; l = ql[jj]; }
+            for (int k = 0; k < kRowsPer; ++k)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t j = j0 + 32 * W * u;
+                    const TA* p = a + min(k, rows - 1) * ld;   // rows past m: not stored
+                    if (VEC && j + W - 1 < n) {
+                        if constexpr (VEC) load4(p + j, x[k][u]);
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < W; ++c) x[k][u][c] = j + c < n ? (V)to_d(__ldcs(p + j + c)) : (V)0;
+                    }
                 }
-                acc_add(acc, x[c], MODE, qd, h, l);
+            double qd[4];
+            float h[4], l[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t jj = j0 + (VEC ? u : 32 * u);
+                qd[u] = 0.0;
+                h[u] = l[u] = 0.f;
+                if (MODE == kDot && jj < n) {
+                    if (F64) qd[u] = q64[jj];
+                    else { h[u] = qh[jj]; l[u] = ql[jj]; }
+                }
             }
+#pragma unroll
+            for (int k = 0; k < kRowsPer; ++k) acc_add4(acc[k], &x[k][0][0], MODE, qd, h, l);
         }
-        const PartT<TA> s = warp_sum_t(part_value(acc));
-        if (lane == 0) out[row] = s;
+#pragma unroll
+        for (int k = 0; k < kRowsPer; ++k) {
+            const PartT<TA> s = warp_sum_t(part_value(acc[k]));
+            if (lane == 0 && k < rows) out[row + k] = s;
+        }
     }
 }
 
@@ -689,8 +860,23 @@ static cur_status launch_pass(const AcaParams& P, int mode, int64_t chunk, int r
                               bool vec, cudaStream_t st) {
     const TA* A = static_cast<const TA*>(P.A);
     PartT<TA>* part = static_cast<PartT<TA>*>(const_cast<void*>(P.part));
+    int dev = 0, sms = 0;
+    CUR_CK(cudaGetDevice(&dev));
+    CUR_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (P.axis == 1) {
         constexpr int TW = 32 * ColsPerLane<TA>::v;
+        if constexpr (!std::is_same<TA, double>::value) {
+            if (vec && ring_pays(kDtypeOf<TA>, P.m, P.n)) {
+                const int64_t coltiles = (P.n + TW - 1) / TW, items = coltiles * rc_count;
+                const size_t sm = (size_t)kRingStages * 32 * TW * sizeof(TA);
+                auto kernel = mode == kNorm ? aca_cols_ring<TA, kNorm> : aca_cols_ring<TA, kDot>;
+                CUR_TRY(smem_attr((const void*)kernel, sm));
+                kernel<<<(unsigned)std::min<int64_t>(3LL * sms, items), 256, sm, st>>>(
+                    A, P.m, P.n, P.ld, chunk, coltiles, items, P.qh, P.ql, part, P.stop);
+                CUR_CK(cudaGetLastError());
+                return CUR_OK;
+            }
+        }
         dim3 grid((unsigned)((P.n + TW - 1) / TW), (unsigned)rc_count);
         if (mode == kNorm) {
             if (vec) aca_cols_pass<TA, kNorm, true><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, chunk, P.q64, P.qh, P.ql, part, P.stop);
@@ -700,15 +886,15 @@ static cur_status launch_pass(const AcaParams& P, int mode, int64_t chunk, int r
             else aca_cols_pass<TA, kDot, false><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, chunk, P.q64, P.qh, P.ql, part, P.stop);
         }
     } else {
-        const int64_t blocks = std::min<int64_t>((P.m + 7) / 8, 65535LL * 8);
-        dim3 grid((unsigned)blocks);
-        if (mode == kNorm) {
-            if (vec) aca_rows_pass<TA, kNorm, true><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
-            else aca_rows_pass<TA, kNorm, false><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
-        } else {
-            if (vec) aca_rows_pass<TA, kDot, true><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
-            else aca_rows_pass<TA, kDot, false><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
-        }
+        const bool four = P.m >= 64LL * sms;
+        const int64_t per = four ? 32 : 8;
+        dim3 grid((unsigned)std::min<int64_t>((P.m + per - 1) / per, 65535LL * 8));
+        auto kernel = mode == kNorm
+            ? (vec ? (four ? aca_rows_pass<TA, kNorm, true, 4> : aca_rows_pass<TA, kNorm, true, 1>)
+                   : (four ? aca_rows_pass<TA, kNorm, false, 4> : aca_rows_pass<TA, kNorm, false, 1>))
+            : (vec ? (four ? aca_rows_pass<TA, kDot, true, 4> : aca_rows_pass<TA, kDot, true, 1>)
+                   : (four ? aca_rows_pass<TA, kDot, false, 4> : aca_rows_pass<TA, kDot, false, 1>));
+        kernel<<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
     }
     CUR_CK(cudaGetLastError());
     return CUR_OK;
@@ -742,18 +928,9 @@ static cur_status aca_run(cur_handle* h, const cur_mat* M, int axis, int r, int3
     P.nsel = axis == 1 ? P.n : P.m;
     P.len = axis == 1 ? P.m : P.n;
     const int G = h->num_sms;
-    // Row chunks of the column pass: enough CTAs for ~32 per SM.
     int RC = 1;
     int64_t chunk = P.m;
-    if (axis == 1) {
-        const int64_t coltiles = (P.n + 32 * ColsPerLane<TA>::v - 1) / (32 * ColsPerLane<TA>::v);
-        int64_t want = std::max<int64_t>(1, (int64_t)h->num_sms * 32 / coltiles);
-        want = std::min<int64_t>(want, std::max<int64_t>(1, P.m / 64));
-        want = std::min<int64_t>(want, 65535);
-        RC = (int)want;
-        chunk = (P.m + RC - 1) / RC;
-        RC = (int)((P.m + chunk - 1) / chunk);
-    }
+    if (axis == 1) RC = aca_cols_chunks(h->num_sms, P.m, P.n, M->dtype, &chunk);
     P.RC = RC;
     P.part = ar.get<double>((size_t)RC * P.nsel);   // PartT is 8 bytes either way
     P.nu = ar.get<double>(P.nsel);
@@ -823,12 +1000,15 @@ cur_status aca_select_full(cur_handle* h, const cur_mat* A, int axis, int r, int
 // ---- the column pass alone, for a row slab of A (the sharded Algorithm 3 in shard.cu)
 
 int aca_cols_chunks(int num_sms, int64_t m, int64_t n, cur_dtype dt, int64_t* chunk) {
+    // items (a column tile of a chunk) for 16 per CTA of the ring's grid, or 32 CTAs per SM of
+    // the direct kernel: the same number; chunks of whole ring stages for a large matrix
     const int cpl = dt == CUR_BF16 ? 8 : 4;
     const int64_t coltiles = (n + 32 * cpl - 1) / (32 * cpl);
     int64_t want = std::max<int64_t>(1, (int64_t)num_sms * 32 / coltiles);
     want = std::min<int64_t>(want, std::max<int64_t>(1, m / 64));
     want = std::min<int64_t>(want, 65535);
-    const int64_t c = (m + want - 1) / want;
+    int64_t c = (m + want - 1) / want;
+    if (curk::ring_pays(dt, m, n)) c = (c + 31) / 32 * 32;
     *chunk = c;
     return (int)((m + c - 1) / c);
 }

@@ -164,13 +164,24 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
                             for (int c = 0; c < 4; ++c) x[u][c] = c0 + c < n ? row[c] : 0.f;
                         }
                     }
+                    if (t >= 0 && i0 + 3 * RG < m) {
+                        float h[4], l[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int64_t i = i0 + RG * u;
-                        if (i >= m) break;
+                        for (int u = 0; u < 4; ++u) { h[u] = qh[i0 + RG * u]; l[u] = ql[i0 + RG * u]; }
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            if (t < 0) acc[c].add_sq(x[u][c]); else acc[c].add(x[u][c], qh[i], ql[i]);
+                            const float xc[4] = {x[0][c], x[1][c], x[2][c], x[3][c]};
+                            acc[c].add4(xc, h, l);
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int64_t i = i0 + RG * u;
+                            if (i >= m) break;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                if (t < 0) acc[c].add_sq(x[u][c]); else acc[c].add(x[u][c], qh[i], ql[i]);
+                            }
                         }
                     }
                 }

@@ -432,14 +432,6 @@ constexpr int kRfB = 128;    // rows and columns of a tile; 8 x 16 threads, 16 x
 constexpr int kRfKC = 32;    // k per stage of W
 constexpr int kRfT = 128;    // threads
 
-__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ uint64_t twice(float x) {
-    uint64_t d;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-    return d;
-}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                  :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -551,11 +543,12 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
             auto step = [&](const ulonglong2* xx, const float2* yy) {
 #pragma unroll
                 for (int b = 0; b < 8; ++b) {
-                    const uint64_t w = twice(b & 1 ? yy[b >> 1].y : yy[b >> 1].x);
+                    const float wf = b & 1 ? yy[b >> 1].y : yy[b >> 1].x;
+                    const uint64_t w = pk(wf, wf);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        fma2(acc[2 * q][b], xx[q].x, w);
-                        fma2(acc[2 * q + 1][b], xx[q].y, w);
+                        acc[2 * q][b] = fma2(xx[q].x, w, acc[2 * q][b]);
+                        acc[2 * q + 1][b] = fma2(xx[q].y, w, acc[2 * q + 1][b]);
                     }
                 }
             };

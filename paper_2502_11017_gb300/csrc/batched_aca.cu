@@ -7,8 +7,8 @@
 // residual nu_j = ||a_j||^2 - sum_k (q_k^T a_j)^2, one read of the matrix per round):
 //   pass   : w_j = a_j^T q_t for every column (Dot2 with q as FP32 hi/lo pairs), the
 //            512 threads split into n/4 four-column groups x as many row groups as fit
-//            (2 for n = 1024, 16 for n = 128), every thread streaming; two CTAs
-//            per SM, so one streams its matrix while the other runs its pivot step
+//            (2 for n = 1024, 16 for n = 128); the rows come through shared memory, one or
+//            two CTAs per SM
 //   pick   : nu_j -= w_j^2, masked argmax (lowest index on ties)
 //   vector : v = a_p - Q W(:,p) with W = the passes' q^T a (the first Gram-Schmidt sweep
 //            needs no Q^T a_p of its own), orthogonalised once more against q_1..q_t
@@ -23,10 +23,11 @@
 #include "common.cuh"
 #include "df64.cuh"
 #include "internal.h"
+#include "tc.cuh"
 
 namespace curk {
 
-constexpr int kBA_T = 512;      // threads per CTA (two CTAs per SM: one streams while the other pivots)
+constexpr int kBA_T = 512;      // threads per CTA
 constexpr int kBA_RG = kBA_T / 256;   // partial-sum rows per column in shared memory: RG n <= kBA_RG kBA_MaxN
 constexpr int kBA_MaxM = 4096;
 constexpr int kBA_MaxN = 1024;
@@ -38,11 +39,22 @@ struct BatAcaItem {
     int64_t joff;             // its J0 at J + joff (r entries)
 };
 
-// shared-memory layout (bytes): nu n x 8 | part RG x n x 8 | v m x 8 | qh m x 4 | ql m x 4 |
-// s kBA_MaxR x 8 | mask n
-__host__ __device__ constexpr size_t bat_aca_smem() {
-    return (size_t)kBA_MaxN * 8 + (size_t)kBA_RG * kBA_MaxN * 8 + (size_t)kBA_MaxM * 8 + (size_t)kBA_MaxM * 8 +
-           (size_t)kBA_MaxR * 8 + kBA_MaxN + 64;
+// The pass's rows on their way: kBA_Slots slots of consecutive rows, of 16 KB each with two CTAs on
+// an SM, of three times that with one. Loaded HBM answers after ~2700 cycles, so an SM's share of it (23
+// bytes per cycle) wants 64 KB in flight; and a slot costs a warp about a hundred instructions beside its
+// sums, so large ones are worth more than a second CTA: 1024 matrices of 2150 x 580 on average take
+// 81 ms with 2 x 3 x 16 KB, 52 with 4 x 32 KB and 48 with 3 x 48 KB.
+constexpr int kBA_Slots = 3;
+constexpr int kBA_Rows = 16384;
+constexpr int bat_slot_bytes(int per_sm) { return (per_sm == 1 ? 3 : 1) * kBA_Rows + 32; }
+constexpr int kBA_Seg = 4;   // row segments of a direction's dot product
+
+// shared-memory layout (bytes): part RG x n x 8 (then the dot products' kBA_Seg x kBA_MaxR x 8) |
+// nu n x 8 | v m x 8 (the direction in the making, then q: high and low words) | s kBA_MaxR x 8 |
+// mask n | ring
+constexpr size_t bat_aca_smem(int per_sm) {
+    return (size_t)kBA_Slots * bat_slot_bytes(per_sm) + (size_t)kBA_RG * kBA_MaxN * 8 + (size_t)kBA_MaxN * 8 + (size_t)kBA_MaxM * 8 +
+           (size_t)kBA_MaxR * 8 + kBA_MaxN;
 }
 
 // (key, index) maximum over the CTA, integer keys (dkey order): no FP64 comparisons.
@@ -71,53 +83,270 @@ __device__ __forceinline__ df64 bat_df_sum(df64 x) {
     return out;
 }
 
-// qs[k] = sum_i Q(k, i) v(i) for k < t (one warp per direction, double-float), then
-// v(i) -= sum_k Q(k, i) qs[k].
-__device__ void bat_project(const float* Qh, const float* Ql, int64_t m, int t, df64* v, df64* qs) {
+// v - sum_{k < t} Q(k, i) qs[k] for the rows ia and ib: the entries of eight directions are loaded
+// before their sums (a chain over k would otherwise wait for memory at each pair), two chains a row.
+__device__ __forceinline__ void bat_minus_q(const float* Qh, const float* Ql, int64_t m, int t, int64_t ia, int64_t ib,
+                                            const df64* qs, df64& va, df64& vb) {
+    constexpr int B = 8;
+    df64 a1{0.f, 0.f}, b1{0.f, 0.f};
+    for (int k0 = 0; k0 < t; k0 += B) {
+        float ha[B], la[B], hb[B], lb[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int64_t o = (int64_t)min(k0 + u, t - 1) * m;   // past t: a valid entry, not used
+            ha[u] = Qh[o + ia];
+            la[u] = Ql[o + ia];
+            hb[u] = Qh[o + ib];
+            lb[u] = Ql[o + ib];
+        }
+#pragma unroll
+        for (int u = 0; u < B; u += 2) {
+            if (k0 + u < t) {
+                const df64 s = qs[k0 + u];
+                va = df_sub(va, df_mul(df64{ha[u], la[u]}, s));
+                vb = df_sub(vb, df_mul(df64{hb[u], lb[u]}, s));
+            }
+            if (k0 + u + 1 < t) {
+                const df64 s = qs[k0 + u + 1];
+                a1 = df_sub(a1, df_mul(df64{ha[u + 1], la[u + 1]}, s));
+                b1 = df_sub(b1, df_mul(df64{hb[u + 1], lb[u + 1]}, s));
+            }
+        }
+    }
+    va = df_add(va, a1);
+    vb = df_add(vb, b1);
+}
+
+// qs[k] = sum_i Q(k, i) v(i) for k < t in double-float: a warp per direction and quarter of the
+// rows (a warp per direction left most of them idle in the last turn, and each waited for eight loads
+// at a time), the quarters in order; then v(i) -= sum_k Q(k, i) qs[k].
+__device__ void bat_project(const float* Qh, const float* Ql, int64_t m, int t, df64* v, df64* qs, df64* seg) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int k = warp; k < t; k += nw) {
+    for (int w = warp; w < kBA_Seg * t; w += nw) {
+        const int k = w / kBA_Seg, g = w % kBA_Seg;
+        const int i0 = (int)(m * g / kBA_Seg), i1 = (int)(m * (g + 1) / kBA_Seg);
         const float* qh = Qh + (int64_t)k * m;
         const float* ql = Ql + (int64_t)k * m;
         df64 a0{0.f, 0.f}, a1{0.f, 0.f};
-        for (int64_t i = lane; i < m; i += 64) {
-            a0 = df_add(a0, df_mul(df64{qh[i], ql[i]}, v[i]));
-            if (i + 32 < m) a1 = df_add(a1, df_mul(df64{qh[i + 32], ql[i + 32]}, v[i + 32]));
+        constexpr int B = 8;
+        for (int i = i0 + lane; i < i1; i += 32 * B) {
+            float h[B], l[B];
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int ii = i + 32 * u < i1 ? i + 32 * u : i;
+                h[u] = qh[ii];
+                l[u] = ql[ii];
+            }
+#pragma unroll
+            for (int u = 0; u < B; u += 2) {
+                const int ia = i + 32 * u, ib = ia + 32;
+                if (ia < i1) a0 = df_add(a0, df_mul(df64{h[u], l[u]}, v[ia]));
+                if (ib < i1) a1 = df_add(a1, df_mul(df64{h[u + 1], l[u + 1]}, v[ib]));
+            }
         }
         df64 s = df_add(a0, a1);
         for (int o = 16; o > 0; o >>= 1)
             s = df_add(s, df64{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)});
-        if (lane == 0) qs[k] = s;
+        if (lane == 0) seg[g * kBA_MaxR + k] = s;
     }
     __syncthreads();
-    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
-        df64 a0{0.f, 0.f}, a1{0.f, 0.f};
-        int k = 0;
-        for (; k + 1 < t; k += 2) {
-            a0 = df_add(a0, df_mul(df64{Qh[(int64_t)k * m + i], Ql[(int64_t)k * m + i]}, qs[k]));
-            a1 = df_add(a1, df_mul(df64{Qh[(int64_t)(k + 1) * m + i], Ql[(int64_t)(k + 1) * m + i]}, qs[k + 1]));
+    for (int k = threadIdx.x; k < t; k += blockDim.x) {
+        df64 s = seg[k];
+        for (int g = 1; g < kBA_Seg; ++g) s = df_add(s, seg[g * kBA_MaxR + k]);
+        qs[k] = s;
+    }
+    __syncthreads();
+    for (int64_t i = threadIdx.x; i < m; i += 2 * blockDim.x) {
+        const int64_t ib = i + blockDim.x;
+        df64 a = v[i], b = ib < m ? v[ib] : df64{0.f, 0.f};
+        bat_minus_q(Qh, Ql, m, t, i, ib < m ? ib : i, qs, a, b);
+        v[i] = a;
+        if (ib < m) v[ib] = b;
+    }
+    __syncthreads();
+}
+
+// Two rows' terms of a thread's four columns (x: row by row; a row left out is zeros).
+template <bool DOT>
+__device__ __forceinline__ void bat_add2(Dot2x2 (&acc)[2], const float (&x)[2][4], df64 q0, df64 q1) {
+    uint64_t y[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const df64 q = u ? q1 : q0;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint64_t a = pk(x[u][2 * k], x[u][2 * k + 1]);
+            y[u][k] = DOT ? acc[k].term(a, pk(q.h, q.h), pk(q.l, q.l)) : acc[k].term_sq(a);
         }
-        if (k < t) a0 = df_add(a0, df_mul(df64{Qh[(int64_t)k * m + i], Ql[(int64_t)k * m + i]}, qs[k]));
-        v[i] = df_sub(v[i], df_add(a0, a1));
     }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) acc[k].c = add2(acc[k].c, add2(y[0][k], y[1][k]));
+}
+
+__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(done) : "r"(su32(b)), "r"(parity) : "memory");
+    return done != 0;
+}
+
+// One round's pass over a matrix: part[rg n + j] = sum over the row group rg's rows i of a_ij q_i
+// (DOT) or a_ij^2. A thread sums the columns cg + cgn c, c = 0..3, of its group's rows: neighbouring
+// lanes take neighbouring words whatever the row's alignment. The rows come by bulk copies of
+// their 16-byte lines, a slot of consecutive rows each; a warp releases a slot when it has summed its
+// part, and no barrier holds the others back. (Loads of every entry to registers: 81 ms for the
+// batch above; 16-byte cp.async with a barrier per slot: 95.) What bounds it is the issue
+// slots: nine FMA-pipe operations per element and about half as many instructions beside the packed sums. Words of the first
+// and last line that lie outside the matrix are not touched. `next` is the slot that fills
+// next and `phase` its parity. False: a copy did not arrive in time.
+template <bool DOT>
+__device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m, int64_t n, int64_t ld, int cgn, int RG,
+                                         const df64* q, unsigned char* ring, int slot_b, uint64_t* bars, uint64_t* freed,
+                                         unsigned& next, unsigned& phase, df64* part) {
+    const int tid = threadIdx.x, cg = tid % cgn, rg = tid / cgn;
+    const bool active = rg < RG;
+    int co[4];   // a column past n: the group's first, its sum is not stored
+#pragma unroll
+    for (int c = 0; c < 4; ++c) co[c] = cg + cgn * c < n ? cg + cgn * c : cg;
+    Dot2x2 acc[2];
+    int per = (int)(kBA_Rows / (ld * 4)) / RG * RG;   // rows per slot
+    if (slot_b > 3 * kBA_Rows && per % (2 * RG) == 0) per *= 3;   // (rows pair up the same way)
+    if (per > 0) {
+        const int stages = (int)((m + per - 1) / per);
+        const uintptr_t base = reinterpret_cast<uintptr_t>(A), end = base + ((m - 1) * ld + n) * 4;
+        auto fill = [&](int s, unsigned slot) {   // thread 0
+            const int64_t r0 = (int64_t)s * per, r1 = min(m, r0 + per);
+            const uintptr_t a0 = base + r0 * ld * 4, a1 = base + ((r1 - 1) * ld + n) * 4;
+            uintptr_t lo = a0 & ~(uintptr_t)15, hi = (a1 + 15) & ~(uintptr_t)15;
+            unsigned char* d = ring + slot * slot_b;
+            const uintptr_t d0 = lo;   // the address at the slot's start
+            if (lo < base) {
+                lo += 16;
+                for (uintptr_t x = a0; x < min(lo, a1); x += 4) *reinterpret_cast<float*>(d + (x - d0)) = *reinterpret_cast<const float*>(x);
+            }
+            if (hi > end) {
+                hi = max(hi - 16, lo);
+                for (uintptr_t x = hi; x < a1; x += 4) *reinterpret_cast<float*>(d + (x - d0)) = *reinterpret_cast<const float*>(x);
+            }
+            hi = max(hi, lo);
+            mbar_expect_tx(&bars[slot], (uint32_t)(hi - lo));
+            if (hi > lo) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                             :: "r"(su32(d + (lo - d0))), "l"(lo), "r"((uint32_t)(hi - lo)), "r"(su32(&bars[slot])) : "memory");
+            }
+        };
+        if (tid == 0)
+            for (int s = 0; s < min(stages, kBA_Slots); ++s) fill(s, (next + s) % kBA_Slots);
+        // addresses by addition only: the loop's issue slots are the sums'
+        const int step = RG * (int)(ld * 4), first = active ? rg * (int)(ld * 4) : 0, bytes = per * (int)(ld * 4);
+        const int o0 = first + 4 * co[0], o1 = first + 4 * co[1], o2 = first + 4 * co[2], o3 = first + 4 * co[3];
+        unsigned slot = next, parity = phase;
+        int shift = (int)(base & 15), left = (int)m;
+        const df64* qr = q + rg;
+        // no barrier of the CTA between slots: a slot is filled again once every warp has released it
+        bool ok = true;
+        unsigned last = 0, last_parity = 0;
+        int s = 0;
+        for (; s < stages; ++s) {
+            ok = __all_sync(0xffffffffu, mbar_try(&bars[slot], parity) || mbar_wait(&bars[slot], parity));
+            if (!ok) break;
+            if (tid == 0 && s > 0 && s - 1 + kBA_Slots < stages && mbar_wait(&freed[last], last_parity)) fill(s - 1 + kBA_Slots, last);
+            if (active) {
+                const unsigned char* f = ring + slot * slot_b + shift;
+                const df64* qs = qr;
+                const int rows = min(per, left);
+                auto row = [&](const unsigned char* x, float (&y)[4]) {
+                    y[0] = *reinterpret_cast<const float*>(x + o0);
+                    y[1] = *reinterpret_cast<const float*>(x + o1);
+                    y[2] = *reinterpret_cast<const float*>(x + o2);
+                    y[3] = *reinterpret_cast<const float*>(x + o3);
+                };
+                int u = rg;
+                for (; u + RG < rows; u += 2 * RG) {
+                    float x[2][4];
+                    row(f, x[0]);
+                    row(f + step, x[1]);
+                    bat_add2<DOT>(acc, x, DOT ? qs[0] : df64{0.f, 0.f}, DOT ? qs[RG] : df64{0.f, 0.f});
+                    f += 2 * step;
+                    qs += 2 * RG;
+                }
+                if (u < rows) {
+                    float x[2][4] = {};
+                    row(f, x[0]);
+                    bat_add2<DOT>(acc, x, DOT ? qs[0] : df64{0.f, 0.f}, df64{0.f, 0.f});
+                }
+            }
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(&freed[slot]);
+            last = slot;
+            last_parity = parity;
+            left -= per;
+            qr += per;
+            shift = (shift + bytes) & 15;
+            if (++slot == kBA_Slots) { slot = 0; parity ^= 1u; }
+        }
+        if (!__syncthreads_and(ok)) {   // wait for the copies in flight, with the same limit, and give up
+            for (int w = s; w < min(stages, s + kBA_Slots); ++w) {
+                mbar_wait(&bars[slot], parity);
+                if (++slot == kBA_Slots) { slot = 0; parity ^= 1u; }
+            }
+            return false;
+        }
+        next = slot;
+        phase = parity;
+    } else if (active) {   // rows too far apart for a slot
+        for (int64_t i = rg; i < m; i += 4 * RG) {
+            float x[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) x[u][c] = i + u * RG < m ? __ldcs(A + (i + u * RG) * ld + co[c]) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 4; u += 2) {
+                const int64_t i0 = min(i + u * RG, m - 1), i1 = min(i + (u + 1) * RG, m - 1);
+                const float y[2][4] = {{x[u][0], x[u][1], x[u][2], x[u][3]}, {x[u + 1][0], x[u + 1][1], x[u + 1][2], x[u + 1][3]}};
+                const df64 z{0.f, 0.f};
+                bat_add2<DOT>(acc, y, DOT ? q[i0] : z, DOT ? q[i1] : z);
+            }
+        }
+    }
+    if (active)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int64_t j = cg + (int64_t)cgn * c;
+            const Dot2 d = acc[c >> 1].half(c & 1);
+            if (j < n) part[rg * n + j] = fast_two_sum(d.s, d.c);
+        }
     __syncthreads();
+    return true;
 }
 
 // order: the matrices by decreasing cost (r m n); queue: a zeroed counter. A CTA takes
 // the next matrix of the order when it finishes one (largest first, so the tail is short).
 __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ data, const BatAcaItem* items,
                                                        const int32_t* order, int* queue, int count, int32_t* J,
-                                                       int32_t* counts, float* Qws, int* status) {
+                                                       int32_t* counts, float* Qws, int slot_b, int* status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double* nu = reinterpret_cast<double*>(smem_raw);
-    df64* part = reinterpret_cast<df64*>(nu + kBA_MaxN);               // RG x n
-    df64* v = part + kBA_RG * kBA_MaxN;                                  // m
-    float* qh = reinterpret_cast<float*>(v + kBA_MaxM);                  // m
-    float* ql = qh + kBA_MaxM;                                           // m
-    df64* qs = reinterpret_cast<df64*>(ql + kBA_MaxM);                   // r
+    df64* part = reinterpret_cast<df64*>(smem_raw);                      // RG x n
+    double* nu = reinterpret_cast<double*>(part + kBA_RG * kBA_MaxN);
+    df64* v = reinterpret_cast<df64*>(nu + kBA_MaxN);                    // m
+    df64* qs = v + kBA_MaxM;                                             // r
     unsigned char* mask = reinterpret_cast<unsigned char*>(qs + kBA_MaxR);
     __shared__ double s_frob2;
     __shared__ int s_next;
+    unsigned char* ring = mask + kBA_MaxN;
+    __shared__ __align__(8) uint64_t bars[kBA_Slots], freed[kBA_Slots];
     const int tid = threadIdx.x;
+    unsigned next = 0, phase = 0;
+    if (tid == 0) {
+        for (int s = 0; s < kBA_Slots; ++s) {
+            mbar_init(&bars[s], 1);
+            mbar_init(&freed[s], kBA_T / 32);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
     float* Qh = Qws + (int64_t)blockIdx.x * 2 * kBA_MaxR * kBA_MaxM;
     float* Ql = Qh + (int64_t)kBA_MaxR * kBA_MaxM;
     // W(t, j) = q_t^T a_j from the passes (the CTA's slice after all CTAs' Q slices)
@@ -135,62 +364,19 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
         const float* A = data + b.aoff;
         const int64_t m = b.m, n = b.n, ld = b.ld;
         const int r = b.r;
-        const bool vec = (n % 4 == 0) && (ld % 4 == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
         // column groups of 4 columns; as many row groups as the CTA's threads cover, so every
         // thread streams (a narrow matrix would otherwise leave most of them idle)
         const int cgn = (int)((n + 3) / 4);
         const int RG = max(1, min((int)blockDim.x / cgn, (int)(kBA_RG * kBA_MaxN / n)));
-        const int cg = tid % cgn, rg = tid / cgn;
-        const bool active = rg < RG;
         for (int j = tid; j < n; j += blockDim.x) mask[j] = 0;
         int picked = 0, bad = 0;
         for (int t = -1; t < r - 1; ++t) {
             // ---- pass: squared norms (t = -1) or w = A^T q_t
-            const int64_t c0 = 4 * (int64_t)cg;
-            Dot2 acc[4];
-            if (active && c0 < n) {
-                // four rows loaded before they are folded: 64 bytes in flight per thread
-                for (int64_t i0 = rg; i0 < m; i0 += 4 * RG) {
-                    float x[4][4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int64_t i = i0 + RG * u;
-                        const float* row = A + (i < m ? i : i0) * ld + c0;
-                        if (vec) {
-                            const float4 y = __ldcs(reinterpret_cast<const float4*>(row));
-                            x[u][0] = y.x; x[u][1] = y.y; x[u][2] = y.z; x[u][3] = y.w;
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) x[u][c] = c0 + c < n ? row[c] : 0.f;
-                        }
-                    }
-                    if (t >= 0 && i0 + 3 * RG < m) {
-                        float h[4], l[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) { h[u] = qh[i0 + RG * u]; l[u] = ql[i0 + RG * u]; }
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float xc[4] = {x[0][c], x[1][c], x[2][c], x[3][c]};
-                            acc[c].add4(xc, h, l);
-                        }
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int64_t i = i0 + RG * u;
-                            if (i >= m) break;
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                if (t < 0) acc[c].add_sq(x[u][c]); else acc[c].add(x[u][c], qh[i], ql[i]);
-                            }
-                        }
-                    }
-                }
+            if (!(t < 0 ? bat_pass<false>(A, m, n, ld, cgn, RG, v, ring, slot_b, bars, freed, next, phase, part)
+                        : bat_pass<true>(A, m, n, ld, cgn, RG, v, ring, slot_b, bars, freed, next, phase, part))) {
+                set_status(status, CUR_ERR_TIMEOUT);
+                return;
             }
-            if (active && c0 < n)
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (c0 + c < n) part[rg * n + c0 + c] = fast_two_sum(acc[c].s, acc[c].c);
-            __syncthreads();
             // ---- pick
             unsigned long long bk = dkey(-INFINITY);
             int bi = INT_MAX;
@@ -229,18 +415,15 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
             const int k = t + 1;
             for (int kk = tid; kk < k; kk += blockDim.x) qs[kk] = W[(int64_t)kk * n + p];
             __syncthreads();
-            for (int64_t i = tid; i < m; i += blockDim.x) {
-                df64 a0{A[i * ld + p], 0.f}, a1{0.f, 0.f};
-                int kk = 0;
-                for (; kk + 1 < k; kk += 2) {
-                    a0 = df_sub(a0, df_mul(df64{Qh[(int64_t)kk * m + i], Ql[(int64_t)kk * m + i]}, qs[kk]));
-                    a1 = df_sub(a1, df_mul(df64{Qh[(int64_t)(kk + 1) * m + i], Ql[(int64_t)(kk + 1) * m + i]}, qs[kk + 1]));
-                }
-                if (kk < k) a0 = df_sub(a0, df_mul(df64{Qh[(int64_t)kk * m + i], Ql[(int64_t)kk * m + i]}, qs[kk]));
-                v[i] = df_add(a0, a1);
+            for (int64_t i = tid; i < m; i += 2 * blockDim.x) {
+                const int64_t ib = i + blockDim.x;
+                df64 a{A[i * ld + p], 0.f}, b{ib < m ? A[ib * ld + p] : 0.f, 0.f};
+                bat_minus_q(Qh, Ql, m, k, i, ib < m ? ib : i, qs, a, b);
+                v[i] = a;
+                if (ib < m) v[ib] = b;
             }
             __syncthreads();
-            bat_project(Qh, Ql, m, k, v, qs);
+            bat_project(Qh, Ql, m, k, v, qs, part);
             df64 nv{0.f, 0.f};
             for (int64_t i = tid; i < m; i += blockDim.x) nv = df_add(nv, df_mul(v[i], v[i]));
             const double s_tot = df_to_d(bat_df_sum(nv));
@@ -257,8 +440,7 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
                 const df64 q = df_mul(v[i], inv);
                 Qh[(int64_t)k * m + i] = q.h;
                 Ql[(int64_t)k * m + i] = q.l;
-                qh[i] = q.h;
-                ql[i] = q.l;
+                v[i] = q;
             }
             __syncthreads();
         }
@@ -278,13 +460,12 @@ size_t bat_aca_workspace(int grid) {
 }
 
 cur_status bat_aca_launch(const float* data, const void* items_dev, const int32_t* order, int* queue, int count,
-                          int32_t* J, int32_t* counts, float* Qws, int grid, int* status, cudaStream_t st) {
+                          int32_t* J, int32_t* counts, float* Qws, int per_sm, int grid, int* status, cudaStream_t st) {
     using namespace curk;
-    const size_t sm = bat_aca_smem();
-    CUR_TRY(smem_attr((const void*)bat_aca_k, sm));
+    CUR_TRY(smem_attr((const void*)bat_aca_k, bat_aca_smem(1)));
     CUR_CK(cudaMemsetAsync(queue, 0, sizeof(int), st));
-    bat_aca_k<<<grid, kBA_T, sm, st>>>(data, static_cast<const BatAcaItem*>(items_dev), order, queue, count, J,
-                                       counts, Qws, status);
+    bat_aca_k<<<grid, kBA_T, bat_aca_smem(per_sm), st>>>(data, static_cast<const BatAcaItem*>(items_dev), order, queue,
+                                                         count, J, counts, Qws, bat_slot_bytes(per_sm), status);
     CUR_CK(cudaGetLastError());
     note_launch();
     return CUR_OK;

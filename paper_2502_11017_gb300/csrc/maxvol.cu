@@ -3008,7 +3008,7 @@ static cur_status bat_global(cur_handle* h, const float* basis, const std::vecto
 size_t bat_aca_workspace(int grid);
 size_t bat_aca_item_size();
 cur_status bat_aca_launch(const float* data, const void* items_dev, const int32_t* order, int* queue, int count,
-                          int32_t* J, int32_t* counts, float* Qws, int grid, int* status, cudaStream_t st);
+                          int32_t* J, int32_t* counts, float* Qws, int per_sm, int grid, int* status, cudaStream_t st);
 
 // The cross of every matrix of the batch (see cur_cross_batched).
 cur_status cross_batched_impl(cur_handle* h, const float* data, const cur_batch_item* items, int T,
@@ -3105,7 +3105,7 @@ cur_status cross_batched_impl(cur_handle* h, const float* data, const cur_batch_
     // ---- J0: Algorithm 3 on the columns of every matrix, padded per matrix
     const int tuned = tune_lookup(h, tkey);
     if (tuned >= 0) {
-        CUR_TRY(bat_aca_launch(data, dai, dorder, queue, T, J0, cnt, Qws, std::min(T, tuned * h->num_sms),
+        CUR_TRY(bat_aca_launch(data, dai, dorder, queue, T, J0, cnt, Qws, tuned, std::min(T, tuned * h->num_sms),
                                h->status, st));
     } else {
         // first batch of this class: time both shapes (each computes the same J0), keep the
@@ -3114,7 +3114,7 @@ cur_status cross_batched_impl(cur_handle* h, const float* data, const cur_batch_
         int best = 2;
         for (int per_sm = 1; per_sm <= 2; ++per_sm) {
             CUR_CK(cudaEventRecord(h->tune_ev[0], st));
-            CUR_TRY(bat_aca_launch(data, dai, dorder, queue, T, J0, cnt, Qws, std::min(T, per_sm * h->num_sms),
+            CUR_TRY(bat_aca_launch(data, dai, dorder, queue, T, J0, cnt, Qws, per_sm, std::min(T, per_sm * h->num_sms),
                                    h->status, st));
             CUR_CK(cudaEventRecord(h->tune_ev[1], st));
             CUR_CK(cudaEventSynchronize(h->tune_ev[1]));

@@ -500,6 +500,32 @@ __device__ __forceinline__ void qsub_pair(const float* Qh, const float* Ql, int6
     acc_b = df_add(acc_b, b1);
 }
 
+// The same for one row by T neighbouring lanes (a power of two): lane h takes the
+// directions h, h + T, ...; all T lanes return the sum.
+template <int T>
+__device__ __forceinline__ df64 qsub_share(const float* Qh, const float* Ql, int64_t len, int k, const df64* s,
+                                           int64_t i, int h, df64 a0) {
+    df64 a1{0.f, 0.f};
+    for (int k0 = h; k0 < k; k0 += kQB * T) {
+        float qh[kQB], ql[kQB];
+#pragma unroll
+        for (int u = 0; u < kQB; ++u) {
+            const int64_t o = (int64_t)min(k0 + u * T, k - 1) * len + i;   // past k: a valid entry, not used
+            qh[u] = Qh[o];
+            ql[u] = Ql[o];
+        }
+#pragma unroll
+        for (int u = 0; u < kQB; u += 2) {
+            if (k0 + u * T < k) a0 = df_sub(a0, df_mul(df64{qh[u], ql[u]}, s[k0 + u * T]));
+            if (k0 + (u + 1) * T < k) a1 = df_sub(a1, df_mul(df64{qh[u + 1], ql[u + 1]}, s[k0 + (u + 1) * T]));
+        }
+    }
+    a0 = df_add(a0, a1);
+#pragma unroll
+    for (int o = T >> 1; o > 0; o >>= 1) a0 = df_add(a0, shfl_xor(a0, o));
+    return a0;
+}
+
 // One round of Algorithm 3 after its pass. `part` holds A^T q_t (t >= 0) or the
 // squared norms (t = -1). Picks index k = t + 1; with `build`, also forms q_k.
 // Cooperative launch; grid G <= co-resident CTAs, block 256. Two group barriers: after
@@ -508,7 +534,7 @@ __device__ __forceinline__ void qsub_pair(const float* Qh, const float* Ql, int6
 // round's barriers wait for bb + G and bb + 2G arrivals (bb = 2 G (t + 1)). A barrier that
 // runs out of time stops the selection, so that no later round waits on a count that
 // cannot be reached.
-template <typename TA>
+template <typename TA, int T>
 __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, int build, unsigned bb) {
     using PT = PartT<TA>;
     __shared__ double s_w[128];
@@ -532,7 +558,37 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
     long long bi = LLONG_MAX;
     double fs = 0.0;
     int bad = 0;
-    {
+    if (T > 1 && P.RC == 1) {   // nothing to add up (a selection of rows): four candidates per thread in flight
+        for (int64_t jb = j0 + tid; jb < j1; jb += 4 * nt) {
+            PT w[4];
+            double old[4];
+            unsigned char picked[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t j = min(jb + u * nt, j1 - 1);
+                w[u] = part[j];
+                old[u] = t < 0 ? 0.0 : P.nu[j];
+                picked[u] = P.mask[j];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t j = jb + u * nt;
+                if (j >= j1) break;
+                const double wd = part_to_d(w[u]);
+                double nu = wd;
+                if (t < 0) {
+                    fs += wd;
+                    if (!isfinite(wd)) bad = 1;
+                } else {
+                    W[(int64_t)t * P.nsel + j] = w[u];
+                    nu = old[u] - wd * wd;
+                }
+                P.nu[j] = nu;
+                const unsigned long long kj = dkey(nu);
+                if (!picked[u] && better_key(kj, (long long)j, bk, bi)) { bk = kj; bi = j; }
+            }
+        }
+    } else {
         const int lane64 = tid & 63, q4 = tid >> 6;   // 64 columns x 4 quarter-sums per pass (first 256 threads)
         for (int64_t jb = j0; jb < j1; jb += 64) {
             const int64_t j = jb + lane64;
@@ -620,6 +676,8 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
     const int64_t len = P.len;
     const int r = P.r;
     const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
+    const int64_t it = i0 + tid / T;   // this thread's row and share, T > 1
+    const int ht = tid % T;
 
     if constexpr (!std::is_same<TA, double>::value) {
         // Double-float form (FP32/BF16 data): the Gram-Schmidt steps on the FP32 pipes;
@@ -637,7 +695,16 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
         // P1b: v = a_p - Q W(:,p), two rows per thread, and this CTA's part of ||v||^2
         {
             df64 nv{0.f, 0.f};
-            for (int64_t ia = i0 + tid; ia < i1; ia += 2 * nt) {
+            if (T > 1 && i0 < i1) {   // rows past i1: computed, not stored (every lane shuffles)
+                const int64_t i = min(it, i1 - 1);
+                const df64 x = qsub_share<T>(Qh, Ql, len, k, s_df, i, ht, df64{ht == 0 ? (float)pivot_elem<TA>(P, i, p) : 0.f, 0.f});
+                if (it < i1 && ht == 0) {
+                    vh[i] = x.h;
+                    vl[i] = x.l;
+                    nv = df_mul(x, x);
+                }
+            }
+            for (int64_t ia = i0 + tid; T == 1 && ia < i1; ia += 2 * nt) {
                 const int64_t ib = ia + nt;
                 const bool vb = ib < i1;
                 df64 acc_a{(float)pivot_elem<TA>(P, ia, p), 0.f};
@@ -707,8 +774,8 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
             const df64 acc0 = warp_sum_t(df_add(a0, a1));
             const df64 acc1 = warp_sum_t(df_add(b0, b1));
             if (lane == 0) {
-                red1[(int64_t)g * r + kk] = acc0;
-                if (two) red1[(int64_t)g * r + kk + 1] = acc1;
+                red1[T > 1 ? (int64_t)kk * G + g : (int64_t)g * r + kk] = acc0;
+                if (two) red1[T > 1 ? (int64_t)(kk + 1) * G + g : (int64_t)g * r + kk + 1] = acc1;
             }
         }
         if (!barrier(2u)) return;
@@ -716,7 +783,42 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
         // same in every CTA): D directions at a time, 256 / D threads per direction each
         // summing every (256 / D)-th CTA with up to kRB loads in flight, then the subsets
         // in order.
-        {
+        // T > 1: a direction's parts lie together and one warp sums them, four directions at a time; the
+        // last warp sums ||v||^2 beside it.
+        const double mx = (double)max(P.m, P.n) * 2.220446049250313e-16;
+        if constexpr (T > 1) {
+            if (warp == nw - 1) {
+                const double vv = warp_sum_strided(P.red2, G);
+                if (lane == 0) s_tot = vv;
+            }
+            constexpr int kD = 4, kL = 5;
+            for (int kb = warp; kb < k; kb += kD * nw) {
+                df64 acc[kD];
+#pragma unroll
+                for (int d = 0; d < kD; ++d) acc[d] = df64{0.f, 0.f};
+                for (int g0 = lane; g0 < G; g0 += 32 * kL) {
+                    df64 x[kD][kL];
+#pragma unroll
+                    for (int d = 0; d < kD; ++d)
+#pragma unroll
+                        for (int u = 0; u < kL; ++u)
+                            x[d][u] = kb + d * nw < k && g0 + 32 * u < G ? red1[(int64_t)(kb + d * nw) * G + g0 + 32 * u]
+                                                                         : df64{0.f, 0.f};
+#pragma unroll
+                    for (int u = 0; u < kL; ++u)
+#pragma unroll
+                        for (int d = 0; d < kD; ++d) acc[d] = df_add(acc[d], x[d][u]);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int d = 0; d < kD; ++d) acc[d] = df_add(acc[d], shfl_xor(acc[d], o));
+#pragma unroll
+                for (int d = 0; d < kD; ++d)
+                    if (lane == 0 && kb + d * nw < k) s_df[kb + d * nw] = acc[d];
+            }
+            __syncthreads();
+        } else {
             constexpr int kRB = 10;
             __shared__ df64 s_sub[kPivotThreads];
             const int D = k <= 32 ? 32 : 64, S = nt / D;
@@ -751,14 +853,13 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
         // first projection, so the difference loses nothing): the early-stop test and the
         // norm of q_k need no further reduction over the CTAs
         if (tid < 32) {
-            const double vv = warp_sum_strided(P.red2, G);
+            const double vv = T > 1 ? s_tot : warp_sum_strided(P.red2, G);
             df64 ss{0.f, 0.f};
             for (int kk = tid; kk < k; kk += 32) ss = df_add(ss, df_mul(s_df[kk], s_df[kk]));
             ss = warp_sum_t(ss);
             if (tid == 0) s_tot = vv - df_to_d(ss);
         }
         __syncthreads();
-        const double mx = (double)max(P.m, P.n) * 2.220446049250313e-16;
         if (!(s_tot > mx * mx * (*P.frob2))) {
             if (g == 0 && tid == 0) { *P.stop = 1; set_status(P.status, CUR_WARN_RANK); }
             return;
@@ -773,7 +874,18 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
         __syncthreads();
         const df64 inv = s_inv;
         // second projection v -= Q s and q_k = v / ||v|| in one sweep
-        for (int64_t ia = i0 + tid; ia < i1; ia += 2 * nt) {
+        if (T > 1 && i0 < i1) {
+            const int64_t i = min(it, i1 - 1);
+            const df64 x = qsub_share<T>(Qh, Ql, len, k, s_df, i, ht, ht == 0 ? df64{vh[i], vl[i]} : df64{0.f, 0.f});
+            if (it < i1 && ht == 0) {
+                const df64 qa = df_mul(x, inv);
+                Qh[(int64_t)k * len + i] = qa.h;
+                Ql[(int64_t)k * len + i] = qa.l;
+                P.qh[i] = qa.h;
+                P.ql[i] = qa.l;
+            }
+        }
+        for (int64_t ia = i0 + tid; T == 1 && ia < i1; ia += 2 * nt) {
             const int64_t ib = ia + nt;
             const bool vb = ib < i1;
             df64 acc_a{vh[ia], vl[ia]};
@@ -853,6 +965,18 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
             P.ql[i] = lo;
         }
     }
+}
+
+// Lanes per row in a pivot's sweeps: few rows per CTA leave its threads idle and the chain over the
+// directions long. 3001 rows on 152 CTAs, a round with 40 directions: 53.5 thousand cycles by one thread per row,
+// 41 by eight lanes (the first sweep 10.3 -> 5.4, the second 7.6 -> 3.1); 2048 rows, 14 directions: 38.5 -> 33.
+// With more than a row per four threads of a CTA one thread per row is the better one (65536 rows: 50 us a round).
+template <typename TA>
+static const void* pivot_kernel(int64_t len, int G) {
+    if constexpr (std::is_same<TA, double>::value) return (const void*)aca_pivot<TA, 1>;   // 28.5 us a round either way
+    const int64_t rows = (len + G - 1) / G;
+    return rows * 8 <= kPivotThreads ? (const void*)aca_pivot<TA, 8>
+           : rows * 4 <= kPivotThreads ? (const void*)aca_pivot<TA, 4> : (const void*)aca_pivot<TA, 1>;
 }
 
 template <typename TA>
@@ -978,7 +1102,7 @@ static cur_status aca_run(cur_handle* h, const cur_mat* M, int axis, int r, int3
         int build = (t + 1 < r - 1) ? 1 : 0;
         unsigned bb = 2u * (unsigned)G * (unsigned)(t + 1);
         void* args[] = {&P, &t, &build, &bb};
-        CUR_TRY(launch_coop((const void*)aca_pivot<TA>, dim3(G), dim3(kPivotThreads), args, 0, st));
+        CUR_TRY(launch_coop(pivot_kernel<TA>(P.len, G), dim3(G), dim3(kPivotThreads), args, 0, st));
         note_launch();
     }
     return CUR_OK;

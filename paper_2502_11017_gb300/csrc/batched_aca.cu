@@ -43,14 +43,12 @@ struct BatAcaItem {
 // an SM, of three times that with one. Loaded HBM answers after ~2700 cycles, so an SM's share of it (23
 // bytes per cycle) wants 64 KB in flight; and a slot costs a warp about a hundred instructions beside its
 // sums, so large ones are worth more than a second CTA: 1024 matrices of 2150 x 580 on average take
-// 81 ms with 2 x 3 x 16 KB, 52 with 4 x 32 KB and 48 with 3 x 48 KB.
+// 81 ms with 2 x 3 x 16 KB, 52 with 4 x 32 KB and 48 with 3 x 48 KB (sums in nine operations; eleven: 53).
 constexpr int kBA_Slots = 3;
 constexpr int kBA_Rows = 16384;
 constexpr int bat_slot_bytes(int per_sm) { return (per_sm == 1 ? 3 : 1) * kBA_Rows + 32; }
-constexpr int kBA_Seg = 4;   // row segments of a direction's dot product
 
-// shared-memory layout (bytes): part RG x n x 8 (then the dot products' kBA_Seg x kBA_MaxR x 8) |
-// nu n x 8 | v m x 8 (the direction in the making, then q: high and low words) | s kBA_MaxR x 8 |
+// shared-memory layout (bytes): part RG x n x 8 | nu n x 8 | v m x 8 (the direction in the making, then q: high and low words) | s kBA_MaxR x 8 |
 // mask n | ring
 constexpr size_t bat_aca_smem(int per_sm) {
     return (size_t)kBA_Slots * bat_slot_bytes(per_sm) + (size_t)kBA_RG * kBA_MaxN * 8 + (size_t)kBA_MaxN * 8 + (size_t)kBA_MaxM * 8 +
@@ -117,70 +115,56 @@ __device__ __forceinline__ void bat_minus_q(const float* Qh, const float* Ql, in
     vb = df_add(vb, b1);
 }
 
-// qs[k] = sum_i Q(k, i) v(i) for k < t in double-float: a warp per direction and quarter of the
-// rows (a warp per direction left most of them idle in the last turn, and each waited for eight loads
-// at a time), the quarters in order; then v(i) -= sum_k Q(k, i) qs[k].
-__device__ void bat_project(const float* Qh, const float* Ql, int64_t m, int t, df64* v, df64* qs, df64* seg) {
+// qs[k] = sum_i Q(k, i) v(i) for k < t (one warp per direction, double-float, sixteen loads in
+// flight per lane), then v(i) -= sum_k Q(k, i) qs[k].
+__device__ void bat_project(const float* Qh, const float* Ql, int64_t m, int t, df64* v, df64* qs) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int w = warp; w < kBA_Seg * t; w += nw) {
-        const int k = w / kBA_Seg, g = w % kBA_Seg;
-        const int i0 = (int)(m * g / kBA_Seg), i1 = (int)(m * (g + 1) / kBA_Seg);
+    for (int k = warp; k < t; k += nw) {
         const float* qh = Qh + (int64_t)k * m;
         const float* ql = Ql + (int64_t)k * m;
         df64 a0{0.f, 0.f}, a1{0.f, 0.f};
         constexpr int B = 8;
-        for (int i = i0 + lane; i < i1; i += 32 * B) {
+        for (int i = lane; i < m; i += 32 * B) {
             float h[B], l[B];
 #pragma unroll
             for (int u = 0; u < B; ++u) {
-                const int ii = i + 32 * u < i1 ? i + 32 * u : i;
+                const int ii = i + 32 * u < m ? i + 32 * u : i;
                 h[u] = qh[ii];
                 l[u] = ql[ii];
             }
 #pragma unroll
             for (int u = 0; u < B; u += 2) {
                 const int ia = i + 32 * u, ib = ia + 32;
-                if (ia < i1) a0 = df_add(a0, df_mul(df64{h[u], l[u]}, v[ia]));
-                if (ib < i1) a1 = df_add(a1, df_mul(df64{h[u + 1], l[u + 1]}, v[ib]));
+                if (ia < m) a0 = df_add(a0, df_mul(df64{h[u], l[u]}, v[ia]));
+                if (ib < m) a1 = df_add(a1, df_mul(df64{h[u + 1], l[u + 1]}, v[ib]));
             }
         }
         df64 s = df_add(a0, a1);
         for (int o = 16; o > 0; o >>= 1)
             s = df_add(s, df64{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)});
-        if (lane == 0) seg[g * kBA_MaxR + k] = s;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < t; k += blockDim.x) {
-        df64 s = seg[k];
-        for (int g = 1; g < kBA_Seg; ++g) s = df_add(s, seg[g * kBA_MaxR + k]);
-        qs[k] = s;
+        if (lane == 0) qs[k] = s;
     }
     __syncthreads();
     for (int64_t i = threadIdx.x; i < m; i += 2 * blockDim.x) {
         const int64_t ib = i + blockDim.x;
-        df64 a = v[i], b = ib < m ? v[ib] : df64{0.f, 0.f};
+        df64 a{0.f, 0.f}, b{0.f, 0.f};
         bat_minus_q(Qh, Ql, m, t, i, ib < m ? ib : i, qs, a, b);
-        v[i] = a;
-        if (ib < m) v[ib] = b;
+        v[i] = df_add(v[i], a);
+        if (ib < m) v[ib] = df_add(v[ib], b);
     }
     __syncthreads();
 }
 
-// Two rows' terms of a thread's four columns (x: row by row; a row left out is zeros).
+// A row's terms of a thread's four columns, in Dot2's eleven operations: the picks of a thousand
+// matrices, some among nearly equal columns, stay those of the scalar sums.
 template <bool DOT>
-__device__ __forceinline__ void bat_add2(Dot2x2 (&acc)[2], const float (&x)[2][4], df64 q0, df64 q1) {
-    uint64_t y[2][2];
+__device__ __forceinline__ void bat_add(Dot2x2 (&acc)[2], const float (&x)[4], df64 q) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const df64 q = u ? q1 : q0;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const uint64_t a = pk(x[u][2 * k], x[u][2 * k + 1]);
-            y[u][k] = DOT ? acc[k].term(a, pk(q.h, q.h), pk(q.l, q.l)) : acc[k].term_sq(a);
-        }
+    for (int k = 0; k < 2; ++k) {
+        const uint64_t a = pk(x[2 * k], x[2 * k + 1]);
+        if (DOT) acc[k].add(a, pk(q.h, q.h), pk(q.l, q.l));
+        else acc[k].c = add2(acc[k].c, acc[k].term_sq(a));
     }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) acc[k].c = add2(acc[k].c, add2(y[0][k], y[1][k]));
 }
 
 __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
@@ -196,7 +180,7 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
 // their 16-byte lines, a slot of consecutive rows each; a warp releases a slot when it has summed its
 // part, and no barrier holds the others back. (Loads of every entry to registers: 81 ms for the
 // batch above; 16-byte cp.async with a barrier per slot: 95.) What bounds it is the issue
-// slots: nine FMA-pipe operations per element and about half as many instructions beside the packed sums. Words of the first
+// slots: eleven FMA-pipe operations per element and about half as many instructions beside the packed sums. Words of the first
 // and last line that lie outside the matrix are not touched. `next` is the slot that fills
 // next and `phase` its parity. False: a copy did not arrive in time.
 template <bool DOT>
@@ -210,7 +194,7 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
     for (int c = 0; c < 4; ++c) co[c] = cg + cgn * c < n ? cg + cgn * c : cg;
     Dot2x2 acc[2];
     int per = (int)(kBA_Rows / (ld * 4)) / RG * RG;   // rows per slot
-    if (slot_b > 3 * kBA_Rows && per % (2 * RG) == 0) per *= 3;   // (rows pair up the same way)
+    if (slot_b > 3 * kBA_Rows) per *= 3;
     if (per > 0) {
         const int stages = (int)((m + per - 1) / per);
         const uintptr_t base = reinterpret_cast<uintptr_t>(A), end = base + ((m - 1) * ld + n) * 4;
@@ -264,17 +248,18 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
                 };
                 int u = rg;
                 for (; u + RG < rows; u += 2 * RG) {
-                    float x[2][4];
-                    row(f, x[0]);
-                    row(f + step, x[1]);
-                    bat_add2<DOT>(acc, x, DOT ? qs[0] : df64{0.f, 0.f}, DOT ? qs[RG] : df64{0.f, 0.f});
+                    float x[4], y[4];
+                    row(f, x);
+                    row(f + step, y);
+                    bat_add<DOT>(acc, x, DOT ? qs[0] : df64{0.f, 0.f});
+                    bat_add<DOT>(acc, y, DOT ? qs[RG] : df64{0.f, 0.f});
                     f += 2 * step;
                     qs += 2 * RG;
                 }
                 if (u < rows) {
-                    float x[2][4] = {};
-                    row(f, x[0]);
-                    bat_add2<DOT>(acc, x, DOT ? qs[0] : df64{0.f, 0.f}, df64{0.f, 0.f});
+                    float x[4];
+                    row(f, x);
+                    bat_add<DOT>(acc, x, DOT ? qs[0] : df64{0.f, 0.f});
                 }
             }
             __syncwarp();
@@ -303,12 +288,8 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
 #pragma unroll
                 for (int c = 0; c < 4; ++c) x[u][c] = i + u * RG < m ? __ldcs(A + (i + u * RG) * ld + co[c]) : 0.f;
 #pragma unroll
-            for (int u = 0; u < 4; u += 2) {
-                const int64_t i0 = min(i + u * RG, m - 1), i1 = min(i + (u + 1) * RG, m - 1);
-                const float y[2][4] = {{x[u][0], x[u][1], x[u][2], x[u][3]}, {x[u + 1][0], x[u + 1][1], x[u + 1][2], x[u + 1][3]}};
-                const df64 z{0.f, 0.f};
-                bat_add2<DOT>(acc, y, DOT ? q[i0] : z, DOT ? q[i1] : z);
-            }
+            for (int u = 0; u < 4; ++u)
+                if (i + u * RG < m) bat_add<DOT>(acc, x[u], DOT ? q[i + u * RG] : df64{0.f, 0.f});
         }
     }
     if (active)
@@ -423,7 +404,7 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
                 if (ib < m) v[ib] = b;
             }
             __syncthreads();
-            bat_project(Qh, Ql, m, k, v, qs, part);
+            bat_project(Qh, Ql, m, k, v, qs);
             df64 nv{0.f, 0.f};
             for (int64_t i = tid; i < m; i += blockDim.x) nv = df_add(nv, df_mul(v[i], v[i]));
             const double s_tot = df_to_d(bat_df_sum(nv));

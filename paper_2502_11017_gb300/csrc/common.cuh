@@ -120,6 +120,23 @@ struct Dot2x2 {
             : "=l"(x), "+l"(s) : "l"(a), "l"(qh), "l"(ql), "l"(kMinus1x2));
         return x;
     }
+    __device__ __forceinline__ void add(uint64_t a, uint64_t qh, uint64_t ql) {   // as Dot2::add
+        asm("{\n\t.reg .b64 p, t, n, u, e;\n\t"
+            "mul.rn.f32x2 p, %2, %3;\n\t"
+            "fma.rn.f32x2 e, p, %5, %6;\n\t"
+            "fma.rn.f32x2 e, %2, %3, e;\n\t"
+            "fma.rn.f32x2 e, %2, %4, e;\n\t"
+            "add.rn.f32x2 t, %0, p;\n\t"
+            "fma.rn.f32x2 n, t, %5, %0;\n\t"     // s - t
+            "add.rn.f32x2 u, t, n;\n\t"
+            "fma.rn.f32x2 u, u, %5, %0;\n\t"     // s - (t + n)
+            "add.rn.f32x2 p, p, n;\n\t"
+            "add.rn.f32x2 u, u, p;\n\t"
+            "add.rn.f32x2 u, u, e;\n\t"
+            "add.rn.f32x2 %1, %1, u;\n\t"
+            "mov.b64 %0, t;\n\t}"
+            : "+l"(s), "+l"(c) : "l"(a), "l"(qh), "l"(ql), "l"(kMinus1x2), "l"(0ull));
+    }
     __device__ __forceinline__ uint64_t term_sq(uint64_t a) {
         uint64_t x;
         asm("{\n\t.reg .b64 p, t, n, u, e;\n\t"

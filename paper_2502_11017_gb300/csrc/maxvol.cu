@@ -1050,6 +1050,9 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
         return sing;
     };
 
+    // M^-1 is carried through the swaps by the first CTA, unless every cycle factorises C(S,:) afresh (FP64 data):
+    // then nothing reads it between (a cross of 2000 x 1500 FP64, r = 16: 2.74 -> 2.66 ms).
+    const bool carry = part == 0 && a.drift_max > 0.0;
     unsigned long long bk;   // argmax |B_ij| as an order key (coef_key), its flat index, a NaN seen
     long long bi;
     int nan;
@@ -1209,10 +1212,8 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
             // the winner's row of B; the first CTA's update of M^-1 runs in four phases
             // between these barriers (see MinvKeeper)
             for (int c = tid; c < r; c += nt) wrow[c] = wsrc[c];
-            if (part == 0) {
-                keep.swap_load(basis + (int64_t)istar * r, r, jstar);
-                if (tid == 0) a.S[(int64_t)pb * rs + jstar] = istar;
-            }
+            if (carry) keep.swap_load(basis + (int64_t)istar * r, r, jstar);
+            if (part == 0 && tid == 0) a.S[(int64_t)pb * rs + jstar] = istar;
             __syncthreads();
             const TB b = wrow[jstar];
             for (int i = tid; i < nloc; i += 4 * nt) {   // four loads in flight (B may be in global memory)
@@ -1223,13 +1224,15 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
                 for (int u = 0; u < 4; ++u)
                     if (i + u * nt < nloc) colj[i + u * nt] = x[u] / b;
             }
-            if (part == 0) keep.swap_partials(r);
+            if (carry) keep.swap_partials(r);
             __syncthreads();
-            if (part == 0) keep.swap_finish_row(r, jstar);
-            __syncthreads();
+            if (carry) {
+                keep.swap_finish_row(r, jstar);
+                __syncthreads();
+            }
             ++made;
             ++total;
-            if (part == 0) keep.swap_update(r, jstar);
+            if (carry) keep.swap_update(r, jstar);
             // B <- B - (B(:,j) / B_ij) (B(i,:) - e_j^T), fused with the next local argmax
             engine_pass<true>(Bs, nloc, r, lo, colj, wrow, jstar, bk, bi, nan);
             par ^= 1;

@@ -450,6 +450,11 @@ cur_status cur_prof_refactors(cur_handle* h, cudaStream_t stream, int64_t* count
  * limit (about 1-2 s in normal calls). */
 cur_status cur_selftest_wait_timeout(cur_handle* h, cudaStream_t stream);
 
+/* The same for the batch's copies: in the handle's next cur_cross_batched the Algorithm 3 launch
+ * withholds those of matrix `item` (the number of matrices or more: of all), so that its waits give
+ * up after ~1 s each. That call records CUR_ERR_TIMEOUT and still returns sets within every matrix. */
+cur_status cur_selftest_batch_timeout(cur_handle* h, int32_t item);
+
 /* Default options: delta 1e-2, max_swaps 100 r, nblocks 1, CUR_FLAG_POLISH. */
 cur_opts cur_default_opts(void);
 

@@ -209,6 +209,12 @@ cur_status cur_selftest_wait_timeout(cur_handle* h, cudaStream_t st) {
     return CUR_OK;
 }
 
+cur_status cur_selftest_batch_timeout(cur_handle* h, int32_t item) {
+    if (!h || item < 0) return CUR_ERR_ARG;
+    h->drop_item = item;
+    return CUR_OK;
+}
+
 cur_status cur_sync_status(cur_handle* h, cudaStream_t st) {
     if (!h) return CUR_ERR_ARG;
     int v = 0;

@@ -182,10 +182,11 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
 // batch above; 16-byte cp.async with a barrier per slot: 95.) What bounds it is the issue
 // slots: eleven FMA-pipe operations per element and about half as many instructions beside the packed sums. Words of the first
 // and last line that lie outside the matrix are not touched. `next` is the slot that fills
-// next and `phase` its parity. False: a copy did not arrive in time.
+// next and `phase` its parity. False: a copy did not arrive in time (`feed` false: none is made, for
+// the self-test).
 template <bool DOT>
 __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m, int64_t n, int64_t ld, int cgn, int RG,
-                                         const df64* q, unsigned char* ring, int slot_b, uint64_t* bars, uint64_t* freed,
+                                         const df64* q, unsigned char* ring, int slot_b, bool feed, uint64_t* bars, uint64_t* freed,
                                          unsigned& next, unsigned& phase, df64* part) {
     const int tid = threadIdx.x, cg = tid % cgn, rg = tid / cgn;
     const bool active = rg < RG;
@@ -220,7 +221,7 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
                              :: "r"(su32(d + (lo - d0))), "l"(lo), "r"((uint32_t)(hi - lo)), "r"(su32(&bars[slot])) : "memory");
             }
         };
-        if (tid == 0)
+        if (tid == 0 && feed)
             for (int s = 0; s < min(stages, kBA_Slots); ++s) fill(s, (next + s) % kBA_Slots);
         // addresses by addition only: the loop's issue slots are the sums'
         const int step = RG * (int)(ld * 4), first = active ? rg * (int)(ld * 4) : 0, bytes = per * (int)(ld * 4);
@@ -304,10 +305,13 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
 }
 
 // order: the matrices by decreasing cost (r m n); queue: a zeroed counter. A CTA takes
-// the next matrix of the order when it finishes one (largest first, so the tail is short).
+// the next matrix of the order when it finishes one (largest first, so the tail is short). A CTA
+// whose wait ran out records it and goes on through the queue without picks: counts and J hold valid
+// entries or -1 for every matrix whatever happens, and the padding and the gathers that follow rely
+// on that. drop: the matrix whose copies are withheld, `count` for all of them, < 0 for none.
 __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ data, const BatAcaItem* items,
                                                        const int32_t* order, int* queue, int count, int32_t* J,
-                                                       int32_t* counts, float* Qws, int slot_b, int* status) {
+                                                       int32_t* counts, float* Qws, int slot_b, int drop, int* status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     df64* part = reinterpret_cast<df64*>(smem_raw);                      // RG x n
     double* nu = reinterpret_cast<double*>(part + kBA_RG * kBA_MaxN);
@@ -320,6 +324,7 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
     __shared__ __align__(8) uint64_t bars[kBA_Slots], freed[kBA_Slots];
     const int tid = threadIdx.x;
     unsigned next = 0, phase = 0;
+    bool lost = false;   // a wait ran out (every thread alike)
     if (tid == 0) {
         for (int s = 0; s < kBA_Slots; ++s) {
             mbar_init(&bars[s], 1);
@@ -351,12 +356,14 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
         const int RG = max(1, min((int)blockDim.x / cgn, (int)(kBA_RG * kBA_MaxN / n)));
         for (int j = tid; j < n; j += blockDim.x) mask[j] = 0;
         int picked = 0, bad = 0;
-        for (int t = -1; t < r - 1; ++t) {
+        const bool feed = drop < 0 || (drop < count && drop != it);
+        for (int t = -1; t < r - 1 && !lost; ++t) {
             // ---- pass: squared norms (t = -1) or w = A^T q_t
-            if (!(t < 0 ? bat_pass<false>(A, m, n, ld, cgn, RG, v, ring, slot_b, bars, freed, next, phase, part)
-                        : bat_pass<true>(A, m, n, ld, cgn, RG, v, ring, slot_b, bars, freed, next, phase, part))) {
+            if (!(t < 0 ? bat_pass<false>(A, m, n, ld, cgn, RG, v, ring, slot_b, feed, bars, freed, next, phase, part)
+                        : bat_pass<true>(A, m, n, ld, cgn, RG, v, ring, slot_b, feed, bars, freed, next, phase, part))) {
                 set_status(status, CUR_ERR_TIMEOUT);
-                return;
+                lost = true;
+                break;
             }
             // ---- pick
             unsigned long long bk = dkey(-INFINITY);
@@ -441,12 +448,13 @@ size_t bat_aca_workspace(int grid) {
 }
 
 cur_status bat_aca_launch(const float* data, const void* items_dev, const int32_t* order, int* queue, int count,
-                          int32_t* J, int32_t* counts, float* Qws, int per_sm, int grid, int* status, cudaStream_t st) {
+                          int32_t* J, int32_t* counts, float* Qws, int per_sm, int grid, int drop, int* status,
+                          cudaStream_t st) {
     using namespace curk;
     CUR_TRY(smem_attr((const void*)bat_aca_k, bat_aca_smem(1)));
     CUR_CK(cudaMemsetAsync(queue, 0, sizeof(int), st));
     bat_aca_k<<<grid, kBA_T, bat_aca_smem(per_sm), st>>>(data, static_cast<const BatAcaItem*>(items_dev), order, queue,
-                                                         count, J, counts, Qws, bat_slot_bytes(per_sm), status);
+                                                         count, J, counts, Qws, bat_slot_bytes(per_sm), drop, status);
     CUR_CK(cudaGetLastError());
     note_launch();
     return CUR_OK;

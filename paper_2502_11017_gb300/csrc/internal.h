@@ -65,6 +65,7 @@ struct cur_handle {
     TuneEntry tune[64] = {};
     int ntune = 0;
     cudaEvent_t tune_ev[2] = {};    // timing events of the tuning runs
+    int drop_item = -1;             // cur_selftest_batch_timeout's matrix, for the next batch
     Arena arena() const {
         Arena a;
         a.base = ws;

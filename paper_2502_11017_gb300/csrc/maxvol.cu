@@ -3011,7 +3011,8 @@ static cur_status bat_global(cur_handle* h, const float* basis, const std::vecto
 size_t bat_aca_workspace(int grid);
 size_t bat_aca_item_size();
 cur_status bat_aca_launch(const float* data, const void* items_dev, const int32_t* order, int* queue, int count,
-                          int32_t* J, int32_t* counts, float* Qws, int per_sm, int grid, int* status, cudaStream_t st);
+                          int32_t* J, int32_t* counts, float* Qws, int per_sm, int grid, int drop, int* status,
+                          cudaStream_t st);
 
 // The cross of every matrix of the batch (see cur_cross_batched).
 cur_status cross_batched_impl(cur_handle* h, const float* data, const cur_batch_item* items, int T,
@@ -3107,9 +3108,11 @@ cur_status cross_batched_impl(cur_handle* h, const float* data, const cur_batch_
     CUR_TRY(bat_upload(h, drr, rr.data(), sizeof(int32_t) * T, st));
     // ---- J0: Algorithm 3 on the columns of every matrix, padded per matrix
     const int tuned = tune_lookup(h, tkey);
+    const int drop = h->drop_item;   // a self-test's, for one call
+    h->drop_item = -1;
     if (tuned >= 0) {
         CUR_TRY(bat_aca_launch(data, dai, dorder, queue, T, J0, cnt, Qws, tuned, std::min(T, tuned * h->num_sms),
-                               h->status, st));
+                               drop, h->status, st));
     } else {
         // first batch of this class: time both shapes (each computes the same J0), keep the
         // faster; this first call waits for the two timed launches
@@ -3118,7 +3121,7 @@ cur_status cross_batched_impl(cur_handle* h, const float* data, const cur_batch_
         for (int per_sm = 1; per_sm <= 2; ++per_sm) {
             CUR_CK(cudaEventRecord(h->tune_ev[0], st));
             CUR_TRY(bat_aca_launch(data, dai, dorder, queue, T, J0, cnt, Qws, per_sm, std::min(T, per_sm * h->num_sms),
-                                   h->status, st));
+                                   drop, h->status, st));
             CUR_CK(cudaEventRecord(h->tune_ev[1], st));
             CUR_CK(cudaEventSynchronize(h->tune_ev[1]));
             float ms = 0.f;

@@ -455,6 +455,11 @@ cur_status cur_selftest_wait_timeout(cur_handle* h, cudaStream_t stream);
  * up after ~1 s each. That call records CUR_ERR_TIMEOUT and still returns sets within every matrix. */
 cur_status cur_selftest_batch_timeout(cur_handle* h, int32_t item);
 
+/* The same for the FP64 inverse of a cluster: four CTAs invert a 64 x 64 matrix, the last step's
+ * message to CTA `lost` (0..2; < 0: to none) withheld. outcomes: 4 int32 (device), what each CTA
+ * returned (0 done, 2 a wait ran out, after ~1 s). */
+cur_status cur_selftest_inverse(cur_handle* h, int32_t lost, int32_t* outcomes, cudaStream_t stream);
+
 /* Default options: delta 1e-2, max_swaps 100 r, nblocks 1, CUR_FLAG_POLISH. */
 cur_opts cur_default_opts(void);
 

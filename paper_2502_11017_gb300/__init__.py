@@ -28,6 +28,7 @@ EXPORTS = ["cur_create", "cur_destroy", "cur_workspace_size", "cur_aca_select", 
            "cur_residual_cheb", "cur_cross", "cur_sync_status", "cur_default_opts",
            "cur_status_string", "cur_prof_enable", "cur_prof_read", "cur_prof_refactors",
            "cur_residual_cheb_noalloc", "cur_selftest_wait_timeout", "cur_selftest_batch_timeout",
+           "cur_selftest_inverse",
            "cur_sketch", "cur_mlp_forward", "cur_mlp_grad", "cur_adam_step", "cur_propose",
            "cur_cross_from", "cur_maxvol_global",
            "cur_shard_aca_state_bytes", "cur_shard_aca_begin", "cur_shard_aca_pick",
@@ -99,6 +100,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         "cur_residual_cheb_noalloc": ([pmat, P, P, P, I32, P, P, P], ctypes.c_int),
         "cur_selftest_wait_timeout": ([P, P], ctypes.c_int),
         "cur_selftest_batch_timeout": ([P, I32], ctypes.c_int),
+        "cur_selftest_inverse": ([P, I32, P, P], ctypes.c_int),
         "cur_prof_read": ([P, P, ctypes.POINTER(D), ctypes.POINTER(I32),
                            ctypes.POINTER(I64)], ctypes.c_int),
         "cur_prof_refactors": ([P, P, ctypes.POINTER(I64)], ctypes.c_int),
@@ -311,6 +313,11 @@ def cur_selftest_wait_timeout(h, stream=None) -> None:
 def cur_selftest_batch_timeout(h, item: int) -> None:
     """Withhold the copies of matrix `item` (a count of matrices: of all) in the next batch."""
     _check(load().cur_selftest_batch_timeout(h, item), "cur_selftest_batch_timeout")
+
+
+def cur_selftest_inverse(h, lost: int, outcomes, stream=None) -> None:
+    """A cluster's inverse with the last message to CTA `lost` withheld; outcomes: 4 int32 on the device."""
+    _check(load().cur_selftest_inverse(h, lost, _ptr(outcomes), _stream(stream)), "cur_selftest_inverse")
 
 
 # ------------------------------------------------------------------ sharded cross (per-rank steps)

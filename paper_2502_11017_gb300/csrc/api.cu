@@ -9,6 +9,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "gj.cuh"
 #include "internal.h"
 
 cur_status pad_indices_dev(int32_t* idx, const int32_t* count, int r, int64_t size, cudaStream_t st);
@@ -27,6 +28,25 @@ __global__ void set_status_k(int* st, int code) {
 // bounded wait must run out, record CUR_ERR_TIMEOUT and return.
 __global__ void selftest_wait_k(unsigned* ctr, int* status, long long limit) {
     group_barrier(ctr, 2u, status, limit);
+}
+
+// The inverse of a 64 x 64 matrix by a cluster of four CTAs (gj.cuh), the last step's message to CTA
+// `mute` withheld (< 0: none); out[rank] = what gj_flow returned there.
+__global__ void __launch_bounds__(32 * kGjWarps) selftest_inverse_k(int mute, int* out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int r = 64;
+    const GjSmem gs(smem_raw, r);
+    const int lane = threadIdx.x & 31;
+    int c0, n;
+    gj_columns(r, 1, c0, n);
+    double v[1][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = lane + 32 * u;
+        v[0][u] = n > 0 ? (i == c0 ? 2.0 : 1.0 / (1 + i + c0)) : 0.0;
+    }
+    const int res = gj_flow<2, 1>(gs, r, 0.0, v, c0, n, nullptr, mute);
+    if (threadIdx.x == 0) out[gj_rank()] = res;
 }
 
 }  // namespace curk
@@ -213,6 +233,11 @@ cur_status cur_selftest_batch_timeout(cur_handle* h, int32_t item) {
     if (!h || item < 0) return CUR_ERR_ARG;
     h->drop_item = item;
     return CUR_OK;
+}
+
+cur_status cur_selftest_inverse(cur_handle* h, int32_t lost, int32_t* outcomes, cudaStream_t st) {
+    if (!h || !outcomes || lost > 2) return CUR_ERR_ARG;
+    return curk::gj_launch(curk::selftest_inverse_k, 4, 4, curk::GjSmem::bytes(64), st, lost, outcomes);
 }
 
 cur_status cur_sync_status(cur_handle* h, cudaStream_t st) {

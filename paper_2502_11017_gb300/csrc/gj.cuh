@@ -97,9 +97,10 @@ __device__ __forceinline__ double gj_row(const double (&v)[RU], int i) {   // en
     return __shfl_sync(0xffffffffu, x, i & 31);
 }
 
-// The pivot of column k (this warp's v, final up to step k - 1), posted to every CTA.
+// The pivot of column k (this warp's v, final up to step k - 1), posted to every CTA (but, for the
+// self-test, the last step's not to CTA `mute`).
 template <int RU>
-__device__ __forceinline__ void gj_post(const GjSmem& s, const double (&v)[RU], int k, int r) {
+__device__ __forceinline__ void gj_post(const GjSmem& s, const double (&v)[RU], int k, int r, int mute) {
     const int lane = threadIdx.x & 31;
     unsigned long long bk = 0ull;
     long long bi = k;
@@ -131,8 +132,9 @@ __device__ __forceinline__ void gj_post(const GjSmem& s, const double (&v)[RU], 
     if (lane == 0) mbar_arrive(&s.bar[k]);
     const unsigned nc = gj_size(), me = gj_rank();
     if (nc == 1) return;
+    auto muted = [&](unsigned q) { return mute >= 0 && k == r - 1 && (int)q == mute; };
     for (unsigned q = 0; q < nc; ++q) {
-        if (q == me) continue;
+        if (q == me || muted(q)) continue;
 #pragma unroll
         for (int u = 0; u < RU; ++u) {
             const int i = lane + 32 * u;
@@ -146,7 +148,7 @@ __device__ __forceinline__ void gj_post(const GjSmem& s, const double (&v)[RU], 
     }
     asm volatile("fence.acq_rel.cluster;" ::: "memory");
     __syncwarp();
-    if ((unsigned)lane < nc && (unsigned)lane != me) gj_arrive(gj_mapa(su32(s.bar + k), (unsigned)lane));
+    if ((unsigned)lane < nc && (unsigned)lane != me && !muted((unsigned)lane)) gj_arrive(gj_mapa(su32(s.bar + k), (unsigned)lane));
 }
 
 // Step k on one column c (RU rows per lane): interchange of rows k and p, elimination.
@@ -166,19 +168,22 @@ __device__ __forceinline__ void gj_step(double (&v)[RU], const double (&ck)[RU],
 // In-place inverse of the matrix whose columns c0 .. c0 + n - 1 this warp holds in v (v[s][u] =
 // row lane + 32 u of column c0 + s; rows past r zero). All threads of every CTA of the cluster
 // call it with 512 threads per CTA. A pivot with !(|pivot| > thresh) ends it: returns 1
-// (singular), 2 after a wait that ran out, else 0; the same value in every thread of a CTA,
-// and of the cluster but for 2. Then column c0 + s belongs at column s.perm[c0 + s] of the inverse.
+// (singular), 2 after a wait that ran out (in any CTA: what the others hold is then not a whole
+// inverse), else 0; the same value in every thread of the cluster. After 0 column c0 + s belongs
+// at column s.perm[c0 + s] of the inverse.
 // logabsdet (may be null): log|det|, in the threads of each CTA's first warp.
 template <int RU, int CPW>
 __device__ __forceinline__ int gj_flow(const GjSmem& s, int r, double thresh, double (&v)[CPW][RU], int c0, int n,
-                                       double* logabsdet) {
+                                       double* logabsdet, int mute = -1) {
     const int lane = threadIdx.x & 31;
+    __shared__ int s_out, s_lost;   // s_lost: a wait ran out in some CTA of the cluster
+    if (threadIdx.x == 0) s_out = s_lost = 0;
     for (int k = threadIdx.x; k < r; k += blockDim.x) mbar_init(&s.bar[k], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
     gj_cluster_sync();
     int out = 0;
-    if (c0 == 0 && n > 0) gj_post<RU>(s, v[0], 0, r);
+    if (c0 == 0 && n > 0) gj_post<RU>(s, v[0], 0, r, mute);
     if (n > 0) {
         for (int k = 0; k < r; ++k) {
             if (!__all_sync(0xffffffffu, gj_wait(&s.bar[k]))) { out = 2; break; }
@@ -198,7 +203,7 @@ __device__ __forceinline__ int gj_flow(const GjSmem& s, int r, double thresh, do
 #pragma unroll
                     for (int u = 0; u < RU; ++u) gj_pick(t[u], v[q][u], q, nx);
                 gj_step<RU>(t, ck, k + 1, k, p, dinv);
-                gj_post<RU>(s, t, k + 1, r);
+                gj_post<RU>(s, t, k + 1, r, mute);
 #pragma unroll
                 for (int q = 0; q < CPW; ++q)
 #pragma unroll
@@ -209,9 +214,6 @@ __device__ __forceinline__ int gj_flow(const GjSmem& s, int r, double thresh, do
                 if (q != nx && q < n) gj_step<RU>(v[q], ck, c0 + q, k, p, dinv);
         }
     }
-    __shared__ int s_out;
-    if (threadIdx.x == 0) s_out = 0;
-    __syncthreads();
     if (out && lane == 0) atomicMax(&s_out, out);
     __syncthreads();
     if (threadIdx.x == 0 && s_out == 0) {   // (a CTA whose warps hold no column follows the messages here)
@@ -246,10 +248,9 @@ __device__ __forceinline__ int gj_flow(const GjSmem& s, int r, double thresh, do
             *logabsdet = acc.log_value();
         }
     }
-    const int res = s_out;
-    __syncthreads();
+    if (threadIdx.x < gj_size() && s_out == 2) gj_st(gj_mapa(su32(&s_lost), threadIdx.x), 1);
     gj_cluster_sync();   // no CTA leaves while another may still write to its shared memory
-    return res;
+    return s_lost ? 2 : s_out;
 }
 
 // CTAs per inverse and columns per warp. A step's FP64 work on one SM is r^2 / 2 clocks, its

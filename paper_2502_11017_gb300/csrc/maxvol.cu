@@ -48,7 +48,8 @@ struct MvProb {
     int64_t base;      // first row of the problem in the basis / B buffers
     int64_t boff;      // element offset of its basis rows (p x r, contiguous)
     int32_t r;         // its rank (<= the stage's r, which is the stride of per-problem arrays)
-    int32_t gmode;     // 1: its B lives in global memory (a problem too large for shared memory)
+    int32_t gmode;     // > 0: its B lives in global memory (a problem too large for shared memory), and C
+                       // passes through shared memory this many rows at a time
     int64_t gid_base;  // global id of local row i = gid_base + i (when gid_arr == null)
     const int32_t* gid_arr;
     int32_t p;         // rows
@@ -559,22 +560,23 @@ constexpr int kMsMax = 64;
 // waiting), and the row CTAs have their shared memory to themselves.
 template <typename TB>
 struct EngineSmem {
-    // rows of C staged per chunk with B in global memory: eight per warp (FP32), or 32
+    // rows of C staged per chunk with B in global memory: eight per warp (FP32), or 32; fewer where
+    // they would not fit beside a slice of many rows (stage_setup). stage = 0: B in shared memory
     static constexpr int kStage = std::is_same<TB, float>::value ? 128 : 32;
     __host__ __device__ static size_t gj(int r) { return ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int); }
-    __host__ __device__ static size_t rows(int nloc, int r, bool gmode) {
-        return gmode ? ((size_t)r * r + nloc + r + 4 + (size_t)kStage * ((r + 3) / 4 * 4)) * sizeof(TB)
+    __host__ __device__ static size_t rows(int nloc, int r, int stage) {
+        return stage ? ((size_t)r * r + nloc + r + 4 + (size_t)stage * ((r + 3) / 4 * 4)) * sizeof(TB)
                      : ((size_t)nloc * r + (size_t)r * r + nloc + r) * sizeof(TB);
     }
     // offset of the MinvKeeper
-    __host__ __device__ static size_t head(int nloc, int r, bool gmode, bool kcta) {
-        const size_t b = kcta ? 0 : rows(nloc, r, gmode);
+    __host__ __device__ static size_t head(int nloc, int r, int stage, bool kcta) {
+        const size_t b = kcta ? 0 : rows(nloc, r, stage);
         return ((b > gj(r) ? b : gj(r)) + 15) / 16 * 16;
     }
-    static size_t bytes(int nloc, int r, bool gmode, bool kcta, bool msm) {
+    static size_t bytes(int nloc, int r, int stage, bool kcta, bool msm) {
         const size_t vec = (size_t)12 * r * sizeof(double) + 64;
-        if (kcta) return std::max(rows(nloc, r, gmode) + 16, head(0, r, gmode, true) + vec + r * sizeof(TB));
-        return head(nloc, r, gmode, false) + vec + (msm ? (size_t)r * r * sizeof(double) : 0);
+        if (kcta) return std::max(rows(nloc, r, stage) + 16, head(0, r, stage, true) + vec + r * sizeof(TB));
+        return head(nloc, r, stage, false) + vec + (msm ? (size_t)r * r * sizeof(double) : 0);
     }
 };
 
@@ -914,10 +916,11 @@ __device__ double engine_kappa(const MinvKeeper<TB>& keep, const TB* basis, cons
 // 8 + 4 TN shared loads per 32 TN FMAs instead of two loads per FMA. Each entry is still one
 // FMA chain over k in order, as a dot product.
 template <int TN, bool GLOB>
-__device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const float* Cs, int nloc, int r, float* area) {
+__device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const float* Cs, int nloc, int r, float* area,
+                                              int stage_rows) {
     constexpr int TM = 8;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    const int chunk = TM * nw, rp = GLOB ? (r + 3) / 4 * 4 : r;
+    const int chunk = GLOB ? min(TM * nw, stage_rows) : TM * nw, rp = GLOB ? (r + 3) / 4 * 4 : r;
     for (int i0 = 0; i0 < nloc; i0 += chunk) {
         const int nr = min(chunk, nloc - i0);
         float* stage = GLOB ? area : Bs + (size_t)i0 * r;
@@ -982,18 +985,28 @@ __device__ __noinline__ void refresh_tiled_tn(float* Bs, const float* Mi, const 
 }
 
 template <bool GLOB>
-__device__ __forceinline__ void engine_refresh_tiled(float* Bs, const float* Mi, const float* Cs, int nloc, int r, float* area) {
+__device__ __forceinline__ void engine_refresh_tiled(float* Bs, const float* Mi, const float* Cs, int nloc, int r, float* area,
+                                                     int stage_rows) {
     switch ((r + 31) / 32) {
-        case 1: refresh_tiled_tn<1, GLOB>(Bs, Mi, Cs, nloc, r, area); break;
-        case 2: refresh_tiled_tn<2, GLOB>(Bs, Mi, Cs, nloc, r, area); break;
-        case 3: refresh_tiled_tn<3, GLOB>(Bs, Mi, Cs, nloc, r, area); break;
-        default: refresh_tiled_tn<4, GLOB>(Bs, Mi, Cs, nloc, r, area);
+        case 1: refresh_tiled_tn<1, GLOB>(Bs, Mi, Cs, nloc, r, area, stage_rows); break;
+        case 2: refresh_tiled_tn<2, GLOB>(Bs, Mi, Cs, nloc, r, area, stage_rows); break;
+        case 3: refresh_tiled_tn<3, GLOB>(Bs, Mi, Cs, nloc, r, area, stage_rows); break;
+        default: refresh_tiled_tn<4, GLOB>(Bs, Mi, Cs, nloc, r, area, stage_rows);
     }
 }
 
 // Problems that one CTA holds alone run with kSoloThreads threads (their swaps never wait on
 // another CTA, so more threads only shorten each swap); groups of CTAs with 256 each.
 constexpr int kSoloThreads = 512;
+
+// Where a group's first CTA has its MinvKeeper. (Not inlined: it is needed once, and inlined it cost
+// the swap loop registers: 56 bytes of stack, 262144 x 64 1.94 -> 1.96 ms.)
+template <typename TB>
+__device__ __noinline__ int keeper_offset(const MvProb& pr, int part) {
+    int lo, nloc;
+    part_rows(pr, part, lo, nloc);
+    return (int)EngineSmem<TB>::head(nloc, pr.r, pr.gmode, pr.kcta && part == 0);
+}
 
 template <typename TB>
 __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
@@ -1008,12 +1021,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
     part_rows(pr, part, lo, nloc);
     const bool gmode = a.bglob != nullptr && pr.gmode;
     const bool keeper = pr.kcta && part == 0;   // this CTA has no rows
-    const size_t off = EngineSmem<TB>::head(nloc, r, gmode, keeper);
     TB* Bs = gmode ? static_cast<TB*>(a.bglob) + pr.boff + (int64_t)lo * r   // nloc x r slice of B
                    : reinterpret_cast<TB*>(smem_raw);
     TB* Mi = gmode ? reinterpret_cast<TB*>(smem_raw) : Bs + (size_t)nloc * r;   // r x r: M^-1 (compute type)
     TB* colj = Mi + (size_t)r * r;              // nloc
-    TB* wrow = keeper ? reinterpret_cast<TB*>(smem_raw + off + (size_t)12 * r * sizeof(double)) : colj + nloc;   // r: winning row of B
+    TB* wrow = keeper ? reinterpret_cast<TB*>(smem_raw + EngineSmem<TB>::head(0, r, 0, true) + (size_t)12 * r * sizeof(double)) : colj + nloc;   // r: winning row of B
     TB* cstage = reinterpret_cast<TB*>((reinterpret_cast<uintptr_t>(wrow + r) + 15) & ~(uintptr_t)15);   // global B: staged C rows
     double* Mg = a.minv64 + (int64_t)pb * minv_stride(rs);      // M^-1 in global memory (FP64)
     __shared__ long long s_w;
@@ -1027,7 +1039,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
     const int myslot = pr.group0 + part;
     if (part == 0) {
         if (tid == 0)
-            keep.setup(smem_raw + off, r, keeper ? static_cast<void*>(smem_raw)
+            keep.setup(smem_raw + keeper_offset<TB>(a.prob[pb], part), r, keeper ? static_cast<void*>(smem_raw)
                                           : pr.msm ? nullptr
                                           : std::is_same<TB, double>::value ? static_cast<void*>(Mg)
                                                                             : static_cast<void*>(a.mdf + (int64_t)pb * 2 * rs * rs));
@@ -1156,10 +1168,10 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
         }
         if constexpr (std::is_same<TB, float>::value) {
             if (!tiled && gmode) {
-                engine_refresh_tiled<true>(Bs, Mi, Cs, nloc, r, cstage);
+                engine_refresh_tiled<true>(Bs, Mi, Cs, nloc, r, cstage, a.prob[pb].gmode);   // (read here: no register held)
                 tiled = true;
             } else if (!tiled && r % 4 == 0 && r >= 32) {
-                engine_refresh_tiled<false>(Bs, Mi, Cs, nloc, r, nullptr);
+                engine_refresh_tiled<false>(Bs, Mi, Cs, nloc, r, nullptr, 0);
                 tiled = true;
             }
         }
@@ -1167,7 +1179,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
             // C rows pass through shared memory a chunk at a time (coalesced loads), then
             // B rows = C rows M^-1 with 8 outputs per thread in registers; the chunk's
             // own rows of Bs serve as the staging area (a separate one when B is global).
-            const int chunk = max(1, min(32, 8 * nt / r));
+            const int chunk = max(1, min(gmode ? a.prob[pb].gmode : 32, 8 * nt / r));
             for (int i0 = 0; i0 < nloc; i0 += chunk) {
                 const int nr = min(chunk, nloc - i0);
                 TB* stage = gmode ? cstage : Bs + (size_t)i0 * r;
@@ -1430,6 +1442,11 @@ __global__ void pad_indices_k(int32_t* idx, const int32_t* count, int r, int64_t
 // 200 KB: a larger slice would leave problems on one CTA that are faster spread (FP64,
 // 1500 x 16 on 24 CTAs). Above, M^-1 and the start's projector leave little room.
 static size_t smem_budget(int r) { return (size_t)(r > kMsMax ? 220 : 200) * 1024; }
+// The most an engine CTA can have: 227 KB less its static arrays (4 KB). With B in global memory a
+// CTA's share of the rows is not bounded by the budget above (a column of B is kept, 4 or 8 bytes a
+// row), so the staged rows give way: 128 rows of them at every size refused 3.7 to 5.1 million rows at
+// r = 128 (FP32) that 32 had taken.
+static const size_t kEngineMost = 223 * 1024;
 static const int kSpreadRows = 64;   // fewest rows per CTA of a spread group
 
 template <typename TB>
@@ -1437,7 +1454,7 @@ static int rows_cap(int r, bool starts, bool kcta) {
     int lo = 1, hi = 1 << 20;
     while (lo < hi) {
         const int mid = (lo + hi + 1) / 2;
-        if ((kcta ? EngineSmem<TB>::bytes(mid, r, false, true, false) : EngineSmem<TB>::bytes(mid, r, false, false, r <= kMsMax)) <= smem_budget(r) &&
+        if ((kcta ? EngineSmem<TB>::bytes(mid, r, 0, true, false) : EngineSmem<TB>::bytes(mid, r, 0, false, r <= kMsMax)) <= smem_budget(r) &&
             (!starts || StartSmem<TB>::bytes(mid, r) <= smem_budget(r))) lo = mid;
         else hi = mid - 1;
     }
@@ -1641,7 +1658,7 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
         // M^-1 has a CTA of its own where it fits no row CTA's shared memory, and where a pass
         // over the group's B in global memory would otherwise wait for the CTA that also
         // updates it
-        pr.msm = pr.r <= kMsMax || EngineSmem<TB>::bytes((int)((pr.p + G - 1) / G), pr.r, pr.gmode != 0, false, true) <= smem_budget(pr.r);
+        pr.msm = pr.r <= kMsMax || EngineSmem<TB>::bytes((int)((pr.p + G - 1) / G), pr.r, pr.gmode ? EngineSmem<TB>::kStage : 0, false, true) <= smem_budget(pr.r);
         pr.kcta = (!pr.msm && !(pr.gmode && many)) || (pr.gmode && G >= 8);
         if (!pr.gmode && (pr.p + cap - 1) / cap > h->num_sms - 1) pr.kcta = 0;   // no SM left for it
         if (pr.kcta) {
@@ -1652,6 +1669,8 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
         G = (pr.p + rpc - 1) / rpc + pr.kcta;
         pr.G = (int)G;
         pr.rpc = rpc;
+        if (pr.gmode) pr.gmode = EngineSmem<TB>::kStage;
+        while (pr.gmode > 8 && EngineSmem<TB>::bytes(rpc, pr.r, pr.gmode, pr.kcta != 0, pr.msm != 0) > kEngineMost) pr.gmode -= 8;
         sg.max_rpc = std::max(sg.max_rpc, rpc);
         anyg |= pr.gmode != 0;
         sg.all_global = sg.all_global && pr.gmode != 0;
@@ -1797,7 +1816,7 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
     size_t sm_eng = 0, sm_start = 0;
     bool wide = false;   // groups with more threads: M^-1 above kMsMax or B in global memory
     for (const auto& pr : sg.probs) {
-        sm_eng = std::max(sm_eng, EngineSmem<TB>::bytes(pr.rpc, pr.r, pr.gmode != 0, pr.kcta != 0, pr.msm != 0));
+        sm_eng = std::max(sm_eng, EngineSmem<TB>::bytes(pr.rpc, pr.r, pr.gmode, pr.kcta != 0, pr.msm != 0));
         wide |= pr.gmode != 0 || pr.kcta != 0;
         sm_start = std::max(sm_start, StartSmem<TB>::bytes(pr.rpc, pr.r));
     }

@@ -177,18 +177,6 @@ __device__ __forceinline__ void store_c_panel(const TcArgs& a, int64_t panel, ui
     tc_fence_before();
 }
 
-// Adds a tile's FP32 sum to a running one: as a double-float (exact to ~2^-48, five FP32
-// operations; in FP64 the two sums of 512 threads took a quarter of the FP64 pipe's time per
-// tile, all on the epilogue's critical path), or in FP64 where its range is needed.
-__device__ __forceinline__ void tc_sum(float x, double& wide, df64& acc) {
-    if (x < 1e28f) {
-        const df64 t = two_sum(acc.h, x);
-        acc = df64{t.h, __fadd_rn(acc.l, t.l)};
-    } else {
-        wide += (double)x;
-    }
-}
-
 // The tiles of one CTA in order: fn(unit, panel group, column tile, panel of the group).
 template <typename F>
 __device__ __forceinline__ void tc_tiles(const TcArgs& a, F&& fn) {
@@ -354,7 +342,6 @@ __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ 
         const uint32_t trow = (uint32_t)(32 * q) << 16;
         float mx = 0.f;
         double se = 0.0, sa = 0.0;
-        df64 sef{0.f, 0.f}, saf{0.f, 0.f};
         int bad = 0;
         int64_t it = 0, seq = 0, cur = -1;
         tc_tiles(a, [&](int64_t, int64_t pg, int64_t, int, int np) {
@@ -411,13 +398,11 @@ __global__ void __launch_bounds__(608, 1) residual_tc_k(const __grid_constant__ 
             const float gs = (s4[0] + s4[1]) + (s4[2] + s4[3]);
             if (gs != gs) bad = 1;
             mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
-            tc_sum(gs, se, sef);
-            tc_sum((a4[0] + a4[1]) + (a4[2] + a4[3]), sa, saf);
+            se += (double)gs;
+            sa += (double)((a4[0] + a4[1]) + (a4[2] + a4[3]));
             ++it;
             return __all_sync(0xffffffffu, abort_flag == 0) != 0;
         });
-        se += df_to_d(sef);
-        sa += df_to_d(saf);
         // reduce over the epilogue threads
         double dmx = mx;
         for (int o = 16; o > 0; o >>= 1) {

@@ -253,15 +253,38 @@ __device__ __forceinline__ int gj_flow(const GjSmem& s, int r, double thresh, do
     return s_lost ? 2 : s_out;
 }
 
-// CTAs per inverse and columns per warp. A step's FP64 work on one SM is r^2 / 2 clocks, its
+inline int gj_cpw(int r, int nc) {   // columns per warp with nc CTAs
+    const int cw = (r + nc - 1) / nc, w = (cw + kGjWarps - 1) / kGjWarps;
+    return w <= 1 ? 1 : (w <= 2 ? 2 : (w <= 4 ? 4 : 8));
+}
+
+// CTAs and columns per warp of a single inverse. A step's FP64 work on one SM is r^2 / 2 clocks, its
 // chain of dependent operations ~600: SMs are added until the work is the shorter (r = 64:
-// four, 128: eight, the portable cluster size), as far as the P problems leave any.
-inline void gj_plan(int r, int P, int num_sms, int* nc, int* cpw) {
+// four, 128: eight, the portable cluster size).
+inline void gj_plan(int r, int* nc, int* cpw) {
     int c = 1;
-    while (c < 8 && r * r > 1200 * c && (int64_t)P * c * 2 <= num_sms) c *= 2;
+    while (c < 8 && r * r > 1200 * c) c *= 2;
     *nc = c;
-    const int cw = (r + c - 1) / c, w = (cw + kGjWarps - 1) / kGjWarps;
-    *cpw = w <= 1 ? 1 : (w <= 2 ? 2 : (w <= 4 ? 4 : 8));
+    *cpw = gj_cpw(r, c);
+}
+
+// CTAs per inverse for a stage of P, 0 for one CTA each with the matrix in shared memory (gj_inverse).
+// Clusters win while all of them run at once; a stage that fills the GPU is bound by the FP64 pipe, which
+// gj_inverse keeps busier (it has no padded columns and fits several CTAs on an SM). us a stage, with
+// clusters of the size taken and with one CTA each in shared memory:
+//   r = 16   P = 152 26 and 32, 1024 108 and 137     r = 32   P = 152 55 and 59, 304 76 and 72, 1024 294 and 254
+//   r = 48   P = 76 83 and 95                        r = 64   P = 36 90 and 140, 76 120 and 140
+//   r = 72   P = 19 140 and 174                      r = 80   P = 36 203 and 230
+//   r = 96   P = 76 328 and 353                      r = 128  P = 16 474 and 726, 76 524 and 726
+// One CTA each in registers is the slower one above r = 32 (r = 64: P = 152 169 and 142, 1024 955 and 763;
+// r = 96: 484 and 351, 3352 and 2051), as are two CTAs at 65 <= r <= 88 (252 and 230 at 80) and four at
+// r <= 74 (162 and 140 at 65). 36 clusters of four run at once, not 38 (r = 96: 247 and 490).
+inline int gj_stage_plan(int r, int P, int num_sms) {
+    if (r <= 32) return r > 24 && P > num_sms ? 0 : 1;
+    if (r > 64 && 8LL * P <= num_sms) return 8;
+    if (r > 48 && (r <= 64 || r > 74) && 4LL * P <= num_sms - 8) return 4;
+    if (r > 34 && (r <= 64 || r > 88) && 2LL * P <= num_sms) return 2;
+    return 0;
 }
 
 // KERNEL<..., RU, CPW> for a rank and a plan; X(RU, CPW) names it.

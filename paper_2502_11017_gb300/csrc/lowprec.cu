@@ -764,7 +764,7 @@ static cur_status lowprec_phase_t(cur_handle* h, const float* C, int64_t p, int 
         lp_quant_c<<<qgrid, 256, 0, st>>>(C, p, r, ldk, static_cast<__nv_bfloat16*>(Cq));
     CUR_CK(cudaGetLastError());
     int nc, cpw;
-    gj_plan(r, 1, h->num_sms, &nc, &cpw);
+    gj_plan(r, &nc, &cpw);
 #define LP_SETUP(RU, CPW) lp_setup_k<F8, RU, CPW>
     CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, LP_SETUP), nc, nc, GjSmem::bytes(r), st, C, r, ldk, S0, S, minv_in, minv_flag,
                       idle, W, winv, Mh, Ml, ctl, gbar));

@@ -457,24 +457,15 @@ __global__ void __launch_bounds__(StartThreads<TB>::v, 1) mv_start(MvArgs a) {
 
 // ---------------------------------------------------------------- FP64 inverse of C(S,:)
 
-// One cluster per problem (gj_plan): a stage of one or a few problems spreads each inverse over
-// up to eight SMs, a stage of many keeps one CTA each. 128 x 128: 717 -> 240 us for one problem,
-// 719 -> 474 us for 16; 1436 -> 1631 us for 256 on one CTA each (FP64-bound either way).
-template <typename TB, int RU, int CPW>
-__global__ void __launch_bounds__(32 * kGjWarps) mv_lu(MvArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const unsigned rank = gj_rank();
-    const int pb = (int)(blockIdx.x / gj_size());
-    if (rank == 0 && threadIdx.x == 0) a.bar[pb] = 0u;   // the swap engine's group barrier starts from zero
-    if (a.done[pb] || !a.lu_mask[pb]) return;
-    const MvProb pr = a.prob[pb];
-    const int r = pr.r, rs = a.r, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    const GjSmem gs(smem_raw, r);
-    __shared__ double s_max;
-    const TB* basis = static_cast<const TB*>(a.basis) + pr.boff;
-    const int32_t* S = a.S + (int64_t)pb * rs;
-    // C(S,:)'s maximum magnitude in the data's type (no FP64 comparisons)
+// The largest magnitude of C(S,:), in the data's type (no FP64 comparisons); -1 where a set or an
+// entry is not usable: that ends the problem, recorded by `first`'s thread 0.
+template <typename TB>
+__device__ __forceinline__ double lu_scale(const MvArgs& a, const MvProb& pr, int pb, const TB* basis, const int32_t* S,
+                                           bool first) {
     using TS = typename std::conditional<std::is_same<TB, double>::value, double, float>::type;
+    __shared__ TS sm[32];
+    __shared__ double s_max;
+    const int r = pr.r, tid = threadIdx.x, nt = blockDim.x;
     TS mx = 0;
     int bad = 0;
     for (int e = tid; e < r * r; e += nt) {
@@ -486,26 +477,39 @@ __global__ void __launch_bounds__(32 * kGjWarps) mv_lu(MvArgs a) {
         mx = fmax(mx, fabs(x));
     }
     bad = __syncthreads_or(bad == 2) ? 2 : (__syncthreads_or(bad == 1) ? 1 : 0);
-    {
-        __shared__ TS sm[32];
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 0) sm[tid >> 5] = mx;
-        __syncthreads();
-        if (tid == 0) {
-            TS t = 0;
-            for (int w = 0; w < (nt >> 5); ++w) t = fmax(t, sm[w]);
-            s_max = (double)t;
-        }
-        __syncthreads();
-    }
-    if (bad) {
-        if (rank == 0 && tid == 0) {
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0) sm[tid >> 5] = mx;
+    __syncthreads();
+    if (tid == 0) {
+        TS t = 0;
+        for (int w = 0; w < (nt >> 5); ++w) t = fmax(t, sm[w]);
+        s_max = (double)t;
+        if (bad && first) {
             a.pstatus[pb] = bad == 2 ? CUR_ERR_NONFINITE : CUR_ERR_ARG;
             a.done[pb] = 1;
             set_status(a.status, bad == 2 ? CUR_ERR_NONFINITE : CUR_ERR_ARG);
         }
-        return;
     }
+    __syncthreads();
+    return bad ? -1.0 : s_max;
+}
+
+// One cluster per problem, its columns in registers (gj.cuh): the form for a stage of few problems,
+// each spread over up to eight SMs (gj_stage_plan has the line and both sides' times).
+template <typename TB, int RU, int CPW>
+__global__ void __launch_bounds__(32 * kGjWarps) mv_lu(MvArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const unsigned rank = gj_rank();
+    const int pb = (int)(blockIdx.x / gj_size());
+    if (rank == 0 && threadIdx.x == 0) a.bar[pb] = 0u;   // the swap engine's group barrier starts from zero
+    if (a.done[pb] || !a.lu_mask[pb]) return;
+    const MvProb pr = a.prob[pb];
+    const int r = pr.r, rs = a.r, tid = threadIdx.x, lane = tid & 31;
+    const GjSmem gs(smem_raw, r);
+    const TB* basis = static_cast<const TB*>(a.basis) + pr.boff;
+    const int32_t* S = a.S + (int64_t)pb * rs;
+    const double scale = lu_scale<TB>(a, pr, pb, basis, S, rank == 0);
+    if (scale < 0.0) return;   // every CTA of the cluster alike
     int c0, n;
     gj_columns(r, CPW, c0, n);
     double v[CPW][RU];
@@ -517,7 +521,7 @@ __global__ void __launch_bounds__(32 * kGjWarps) mv_lu(MvArgs a) {
             v[q][u] = q < n && i < r ? (double)basis[(int64_t)S[i] * r + c0 + q] : 0.0;
         }
     double lv = 0.0;
-    const int res = gj_flow<RU, CPW>(gs, r, (double)r * kEps * s_max, v, c0, n, &lv);
+    const int res = gj_flow<RU, CPW>(gs, r, (double)r * kEps * scale, v, c0, n, &lv);
     if (res) {
         if (rank == 0 && tid == 0) {
             a.pstatus[pb] = res == 2 ? CUR_ERR_TIMEOUT : CUR_ERR_SINGULAR;
@@ -542,6 +546,39 @@ __global__ void __launch_bounds__(32 * kGjWarps) mv_lu(MvArgs a) {
                 if (i < r) out64[(int64_t)i * r + c] = v[q][u];
             }
         }
+}
+
+// One CTA per problem, the matrix in shared memory (gj_inverse): the form for a stage whose problems
+// fill the GPU. The same inverses to the bit.
+template <typename TB>
+__global__ void __launch_bounds__(512) mv_lu_cta(MvArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int pb = blockIdx.x;
+    if (threadIdx.x == 0) a.bar[pb] = 0u;   // the swap engine's group barrier starts from zero
+    if (a.done[pb] || !a.lu_mask[pb]) return;
+    const MvProb pr = a.prob[pb];
+    const int r = pr.r, rs = a.r, tid = threadIdx.x, nt = blockDim.x;
+    double* M = reinterpret_cast<double*>(smem_raw);  // r x r, inverted in place
+    double* colk = M + r * r;
+    int* piv = reinterpret_cast<int*>(colk + r);
+    const TB* basis = static_cast<const TB*>(a.basis) + pr.boff;
+    const int32_t* S = a.S + (int64_t)pb * rs;
+    const double scale = lu_scale<TB>(a, pr, pb, basis, S, true);
+    if (scale < 0.0) return;
+    for (int e = tid; e < r * r; e += nt) M[e] = (double)basis[(int64_t)S[e / r] * r + e % r];
+    __syncthreads();
+    double lv = 0.0;
+    const int sing = gj_inverse(M, r, colk, piv, (double)r * kEps * scale, &lv);
+    if (sing) {
+        if (tid == 0) { a.pstatus[pb] = CUR_ERR_SINGULAR; a.done[pb] = 1; a.logvol[pb] = -INFINITY; }
+        return;
+    }
+    double* out64 = a.minv64 + (int64_t)pb * minv_stride(rs);
+    for (int e = tid; e < r * r; e += nt) out64[e] = M[e];
+    if (tid == 0) {
+        a.logvol[pb] = lv;
+        out64[r * r] = 0.0;   // fresh: no drift
+    }
 }
 
 // ---------------------------------------------------------------- the swap iteration
@@ -1863,11 +1900,16 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
             note_launch();
         }
     }
-    {
-        int nc, cpw;
-        gj_plan(r, P, h->num_sms, &nc, &cpw);
+    const int nc = gj_stage_plan(r, P, h->num_sms);
+    if (nc == 0) {
+        const size_t sm_lu = ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int) + 64;
+        CUR_TRY(smem_attr((const void*)mv_lu_cta<TB>, sm_lu));
+        mv_lu_cta<TB><<<P, 512, sm_lu, st>>>(a);
+        CUR_CK(cudaGetLastError());
+        note_launch();
+    } else {
 #define MV_LU(RU, CPW) mv_lu<TB, RU, CPW>
-        CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, MV_LU), P * nc, nc, GjSmem::bytes(r), st, a));
+        CUR_TRY(gj_launch(GJ_KERNEL(r, gj_cpw(r, nc), MV_LU), P * nc, nc, GjSmem::bytes(r), st, a));
 #undef MV_LU
     }
     if (sg.bpre) {

@@ -700,7 +700,7 @@ static cur_status assemble_t(cur_handle* h, const cur_mat* Am, const int32_t* I,
     note_launch();
     }
     int nc, cpw;
-    gj_plan(r, 1, h->num_sms, &nc, &cpw);
+    gj_plan(r, &nc, &cpw);
 #define ASSEMBLE(RU, CPW) assemble_gj_k<TA, RU, CPW>
     CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, ASSEMBLE), nc, nc, GjSmem::bytes(r), st, A, Am->rows, Am->cols, Am->ld, I, J, r,
                       U_out, rcond_out, work, redo));

@@ -50,11 +50,6 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float v[4]) {
     v[2] = __uint_as_float(x.y << 16);
     v[3] = __uint_as_float(x.y & 0xffff0000u);
 }
-template <typename TA, typename TV>
-__device__ __forceinline__ void load4_guard(const TA* row, int64_t col, int64_t n, TV v[4]) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = (col + k < n) ? (TV)to_d(row[col + k]) : (TV)0;
-}
 
 // Columns per lane of the column pass: 16 bytes of A per lane and row (8 for BF16).
 template <typename TA> struct ColsPerLane { static constexpr int v = sizeof(TA) == 2 ? 8 : 4; };
@@ -973,10 +968,13 @@ __global__ void __launch_bounds__(kPivotThreads) aca_pivot(AcaParams P, int t, i
 // With more than a row per four threads of a CTA one thread per row is the better one (65536 rows: 50 us a round).
 template <typename TA>
 static const void* pivot_kernel(int64_t len, int G) {
-    if constexpr (std::is_same<TA, double>::value) return (const void*)aca_pivot<TA, 1>;   // 28.5 us a round either way
-    const int64_t rows = (len + G - 1) / G;
-    return rows * 8 <= kPivotThreads ? (const void*)aca_pivot<TA, 8>
-           : rows * 4 <= kPivotThreads ? (const void*)aca_pivot<TA, 4> : (const void*)aca_pivot<TA, 1>;
+    if constexpr (std::is_same<TA, double>::value) {
+        return (const void*)aca_pivot<TA, 1>;   // 28.5 us a round either way
+    } else {
+        const int64_t rows = (len + G - 1) / G;
+        return rows * 8 <= kPivotThreads ? (const void*)aca_pivot<TA, 8>
+               : rows * 4 <= kPivotThreads ? (const void*)aca_pivot<TA, 4> : (const void*)aca_pivot<TA, 1>;
+    }
 }
 
 template <typename TA>

@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
             }
             if (kk < kc) step(x, y);
         }
-        const bool whole = c0 + kRfB <= n && pairs;
+        const bool whole = pairs && c0 + kRfB <= n;
 #pragma unroll
         for (int grp = 0; grp < 2; ++grp) {
             float tmx = 0.f, tse = 0.f, tsa = 0.f;
@@ -600,17 +600,31 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
                             fold(__uint_as_float(bits), __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)));
                         }
                 } else {
+                    // A's last rows or columns, or rows off the pairs' grid: one element per load, the
+                    // 32 loads issued before they are folded, and an entry past A's end folds as zeros
+                    // (loaded and folded one by one: BF16 113763 x 393, r = 16, 240 us; residual_k 169,
+                    // this 147). BF16 loads some valid address instead of a predicate: its conversions
+                    // otherwise wait for each load in turn (259 us); FP32 is faster with one (124 and 148)
+                    TA raw[4][8];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
-                        if (i0 + a >= m) break;
+                        const TA* p = A + min(i0 + a, m - 1) * ld;
 #pragma unroll
                         for (int b = 0; b < 8; ++b) {
                             const int64_t col = c0 + 2 * tx + 32 * (b >> 1) + (b & 1);
-                            const int row = grp * 8 + a0 + a;
-                            const uint64_t d = acc[row >> 1][b];
-                            if (col < n) fold(to_f(A[(i0 + a) * ld + col]), __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)));
+                            if constexpr (sizeof(TA) == 4) raw[a][b] = i0 + a < m && col < n ? p[col] : 0.f;
+                            else raw[a][b] = p[col < n ? col : 0];
                         }
                     }
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+#pragma unroll
+                        for (int b = 0; b < 8; ++b) {
+                            const int row = grp * 8 + a0 + a;
+                            const uint64_t d = acc[row >> 1][b];
+                            const bool in = i0 + a < m && c0 + 2 * tx + 32 * (b >> 1) + (b & 1) < n;
+                            fold(in ? to_f(raw[a][b]) : 0.f, in ? __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)) : 0.f);
+                        }
                 }
             }
             mx = fmax(mx, (double)tmx);

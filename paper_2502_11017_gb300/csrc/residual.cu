@@ -45,7 +45,7 @@ __global__ void gather_R_k(const TA* __restrict__ A, int64_t m, int64_t n, int64
     }
 }
 
-// The usual case of the assembly: U = A(I,J)^-1 in FP64 by one cluster (gj.cuh), its rcond in
+// The usual case of the assembly above r = 44: U = A(I,J)^-1 in FP64 by one cluster (gj.cuh), its rcond in
 // the 1-norm. Where the inverse does not stand (a singular or ill-conditioned M, indices out of
 // range, data that are not finite) *redo is set and assemble_inv_k decides. colsum: r doubles.
 // r = 128: 1220 us in assemble_inv_k.
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(32 * kGjWarps) assemble_gj_k(const TA* __restr
     }
 }
 
-// Where *redo is set, one CTA: M = A(I,J) in FP64, LU with partial pivoting, inverse, rcond; if
+// Where *redo is set (or redo is null: always), one CTA: M = A(I,J) in FP64, LU with partial pivoting, inverse, rcond; if
 // rcond < 1e-13 (or M is singular) the pseudo-inverse from a one-sided Jacobi SVD
 // (round-robin pair order, one warp per pair) with cutoff r eps s_max.
 // work: 3 r^2 doubles (global scratch).
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256) assemble_inv_k(const TA* __restrict__ A, 
                                                       double* __restrict__ work, int* status,
                                                       const int* __restrict__ redo) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (!*redo) return;
+    if (redo && !*redo) return;
     const int tid = threadIdx.x, nt = blockDim.x;
     double* M = reinterpret_cast<double*>(smem_raw);  // r x r, inverted in place
     double* colk = M + r * r;
@@ -713,12 +713,19 @@ static cur_status assemble_t(cur_handle* h, const cur_mat* Am, const int32_t* I,
         CUR_CK(cudaGetLastError());
     note_launch();
     }
-    int nc, cpw;
-    gj_plan(r, &nc, &cpw);
+    // Up to r = 44 assemble_inv_k alone is the faster (us an assembly of 600 x 500, with assemble_gj_k
+    // before it and alone: r = 4 26.7 and 22.6, 16 43.0 and 39.0, 33 86 and 68, 44 98.3 and 96.4, 48 106 and
+    // 117, 64 112 and 209): a cluster's launch, and the second kernel's that then finds nothing to do
+    if (r > 44) {
+        int nc, cpw;
+        gj_plan(r, &nc, &cpw);
 #define ASSEMBLE(RU, CPW) assemble_gj_k<TA, RU, CPW>
-    CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, ASSEMBLE), nc, nc, GjSmem::bytes(r), st, A, Am->rows, Am->cols, Am->ld, I, J, r,
-                      U_out, rcond_out, work, redo));
+        CUR_TRY(gj_launch(GJ_KERNEL(r, cpw, ASSEMBLE), nc, nc, GjSmem::bytes(r), st, A, Am->rows, Am->cols, Am->ld, I, J, r,
+                          U_out, rcond_out, work, redo));
 #undef ASSEMBLE
+    } else {
+        redo = nullptr;
+    }
     const size_t sm = ((size_t)r * r + r) * sizeof(double) + (size_t)r * sizeof(int) + 64;
     CUR_TRY(smem_attr((const void*)assemble_inv_k<TA>, sm));
     assemble_inv_k<TA><<<1, 256, sm, st>>>(A, Am->rows, Am->cols, Am->ld, I, J, r, U_out, rcond_out, work, h->status, redo);

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(256, 3) aca_cols_ring(const TA* __restrict__ A
 }
 
 // out[i] = sum_j a_ij * q_j (kDot) or a_ij^2 (kNorm); one warp per kRowsPer rows (4, or 1
-// below two CTAs per SM), so that each entry of q serves that many loads of A. VEC: four consecutive columns per lane (16 bytes of
+// below two CTAs per SM and for FP64: 65536 x 8192 7.40 ms a selection of 8 with one, 7.67 with four), so that each entry of q serves that many loads of A. VEC: four consecutive columns per lane (16 bytes of
 // FP32); else lane l takes the columns l, l + 32, ...: 128-byte runs whatever the alignment (one
 // 4-byte access per row; four strided by lane, each touching every line, took 92 us a pass at
 // 20001 x 3001 FP32 (2.6 TB/s), this 61).
@@ -409,6 +409,50 @@ __global__ void __launch_bounds__(256) aca_rows_pass(const TA* __restrict__ A, i
             if (lane == 0 && k < rows) out[row + k] = s;
         }
     }
+}
+
+// The same, one row per warp, four consecutive columns per lane and the terms one by one: for FP64 and
+// BF16 where that is the faster (rows_each).
+template <typename TA, int MODE, bool VEC>
+__global__ void __launch_bounds__(256) aca_rows_each(const TA* __restrict__ A, int64_t m, int64_t n, int64_t ld,
+                                                     const double* __restrict__ q64, const float* __restrict__ qh,
+                                                     const float* __restrict__ ql, PartT<TA>* __restrict__ out,
+                                                     const int* __restrict__ stop) {
+    using V = typename ValT<TA>::type;
+    constexpr bool F64 = std::is_same<TA, double>::value;
+    if (*stop) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int64_t row = (int64_t)blockIdx.x * 8 + warp; row < m; row += (int64_t)gridDim.x * 8) {
+        const TA* a = A + row * ld;
+        AccOf<TA> acc;
+        for (int64_t j = (int64_t)lane * 4; j < n; j += 128) {
+            V x[4];
+            if (VEC && j + 3 < n) load4(a + j, x); else loadc_guard<4>(a, j, n, x);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                double qd = 0.0;
+                float h = 0.f, l = 0.f;
+                if (MODE == kDot && j + c < n) {
+                    if (F64) qd = q64[j + c];
+                    else { h = qh[j + c]; l = ql[j + c]; }
+                }
+                acc_add(acc, x[c], MODE, qd, h, l);
+            }
+        }
+        const PartT<TA> s = warp_sum_t(part_value(acc));
+        if (lane == 0) out[row] = s;
+    }
+}
+
+// Whether rows go one by one (us a selection of 8: one by one, aca_rows_pass with one row, with four):
+//   BF16: four rows' 8-byte loads bring too little each, and nine operations per term in fours wait
+//   longer than eleven one by one where there are few warps. By vectors 600 x 8192 369, 382, 750;
+//   9000 x 8192 776, 715, 1289; 10000 x 8192 823, 888, 1282; 65536 x 8192 3758, 3700, 5428. Off the 16-byte
+//   grid 600 x 8191 365, 475, 592; 5500 x 4095 410, 434; 9000 x 2047 342, 300, 310; 65536 x 8191 4603, 3515, 3016.
+//   FP64 off the grid, in L2: 600 x 8191 366, 480; 1000 x 4095 271, 333; 1500 x 4095 324, 343; but 3000 x 8191 676, 590.
+static bool rows_each(cur_dtype dt, bool vec, int64_t m, int sms) {
+    if (dt == CUR_F64) return !vec && m < 16LL * sms;
+    return dt == CUR_BF16 && (m < 40LL * sms || (vec && m >= 64LL * sms));
 }
 
 struct AcaParams {
@@ -1008,14 +1052,26 @@ static cur_status launch_pass(const AcaParams& P, int mode, int64_t chunk, int r
             else aca_cols_pass<TA, kDot, false><<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, chunk, P.q64, P.qh, P.ql, part, P.stop);
         }
     } else {
-        const bool four = P.m >= 64LL * sms;
+        constexpr bool F64 = std::is_same<TA, double>::value;
+        constexpr int kMany = F64 ? 1 : 4;
+        const bool each = rows_each(kDtypeOf<TA>, vec, P.m, sms);
+        const bool four = !F64 && !each && P.m >= 64LL * sms;
         const int64_t per = four ? 32 : 8;
         dim3 grid((unsigned)std::min<int64_t>((P.m + per - 1) / per, 65535LL * 8));
+        if constexpr (!std::is_same<TA, float>::value) {
+            if (each) {
+                auto kernel = mode == kNorm ? (vec ? aca_rows_each<TA, kNorm, true> : aca_rows_each<TA, kNorm, false>)
+                                            : (vec ? aca_rows_each<TA, kDot, true> : aca_rows_each<TA, kDot, false>);
+                kernel<<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
+                CUR_CK(cudaGetLastError());
+                return CUR_OK;
+            }
+        }
         auto kernel = mode == kNorm
-            ? (vec ? (four ? aca_rows_pass<TA, kNorm, true, 4> : aca_rows_pass<TA, kNorm, true, 1>)
-                   : (four ? aca_rows_pass<TA, kNorm, false, 4> : aca_rows_pass<TA, kNorm, false, 1>))
-            : (vec ? (four ? aca_rows_pass<TA, kDot, true, 4> : aca_rows_pass<TA, kDot, true, 1>)
-                   : (four ? aca_rows_pass<TA, kDot, false, 4> : aca_rows_pass<TA, kDot, false, 1>));
+            ? (vec ? (four ? aca_rows_pass<TA, kNorm, true, kMany> : aca_rows_pass<TA, kNorm, true, 1>)
+                   : (four ? aca_rows_pass<TA, kNorm, false, kMany> : aca_rows_pass<TA, kNorm, false, 1>))
+            : (vec ? (four ? aca_rows_pass<TA, kDot, true, kMany> : aca_rows_pass<TA, kDot, true, 1>)
+                   : (four ? aca_rows_pass<TA, kDot, false, kMany> : aca_rows_pass<TA, kDot, false, 1>));
         kernel<<<grid, 256, 0, st>>>(A, P.m, P.n, P.ld, P.q64, P.qh, P.ql, part, P.stop);
     }
     CUR_CK(cudaGetLastError());

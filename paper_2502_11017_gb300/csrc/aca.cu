@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(256) aca_cols_pass(const TA* __restrict__ A, i
     using V = typename ValT<TA>::type;
     using PT = PartT<TA>;
     constexpr int CPL = ColsPerLane<TA>::v, TW = 32 * CPL;
+    constexpr bool F64 = std::is_same<TA, double>::value;
     __shared__ PT red[8][TW];
     if (*stop) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -142,21 +143,32 @@ __global__ void __launch_bounds__(256) aca_cols_pass(const TA* __restrict__ A, i
     int64_t i = r0 + warp;
     for (; i + 24 < r1; i += 32) {
         V x[4][CPL];
-        double qd[4];
-        float h[4], l[4];
+        if constexpr (F64) {   // row by row, each entry of q when its row is summed (1000 x 1001: 197 us a
+                               // selection of 8, by columns as below 213)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const TA* row = A + (i + 8 * u) * ld;
-            if (full) loadc(row + col, x[u]); else loadc_guard<CPL>(row, col, n, x[u]);
-            if (MODE == kDot) {
-                if (std::is_same<TA, double>::value) qd[u] = q64[i + 8 * u];
-                else { h[u] = qh[i + 8 * u]; l[u] = ql[i + 8 * u]; }
+            for (int u = 0; u < 4; ++u) {
+                const TA* row = A + (i + 8 * u) * ld;
+                if (full) loadc(row + col, x[u]); else loadc_guard<CPL>(row, col, n, x[u]);
             }
-        }
 #pragma unroll
-        for (int c = 0; c < CPL; ++c) {
-            const V xc[4] = {x[0][c], x[1][c], x[2][c], x[3][c]};
-            acc_add4(acc[c], xc, MODE, qd, h, l);
+            for (int u = 0; u < 4; ++u) {
+                const double qd = MODE == kDot ? q64[i + 8 * u] : 0.0;
+#pragma unroll
+                for (int c = 0; c < CPL; ++c) acc_add(acc[c], x[u][c], MODE, qd, 0.f, 0.f);
+            }
+        } else {
+            float h[4], l[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const TA* row = A + (i + 8 * u) * ld;
+                if (full) loadc(row + col, x[u]); else loadc_guard<CPL>(row, col, n, x[u]);
+                if (MODE == kDot) { h[u] = qh[i + 8 * u]; l[u] = ql[i + 8 * u]; }
+            }
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                const V xc[4] = {x[0][c], x[1][c], x[2][c], x[3][c]};
+                acc_add4(acc[c], xc, MODE, nullptr, h, l);
+            }
         }
     }
     for (; i < r1; i += 8) {
@@ -1179,14 +1191,20 @@ cur_status aca_select_full(cur_handle* h, const cur_mat* A, int axis, int r, int
 
 int aca_cols_chunks(int num_sms, int64_t m, int64_t n, cur_dtype dt, int64_t* chunk) {
     // items (a column tile of a chunk) for 16 per CTA of the ring's grid, or 32 CTAs per SM of
-    // the direct kernel: the same number; chunks of whole ring stages for a large matrix
+    // the direct kernel: the same number; chunks of whole ring stages for a large matrix, at least
+    // four where that leaves every CTA of the ring an item: an item ends with two barriers and the
+    // sum over 8 warps (us a selection of 8 FP32, by the direct kernel and by the ring with chunks of 64,
+    // 96 and 128 rows: 65536 x 512 573, 621, 535, 500; 4096 x 8192 392, 414, 394, 386)
     const int cpl = dt == CUR_BF16 ? 8 : 4;
     const int64_t coltiles = (n + 32 * cpl - 1) / (32 * cpl);
     int64_t want = std::max<int64_t>(1, (int64_t)num_sms * 32 / coltiles);
     want = std::min<int64_t>(want, std::max<int64_t>(1, m / 64));
     want = std::min<int64_t>(want, 65535);
     int64_t c = (m + want - 1) / want;
-    if (curk::ring_pays(dt, m, n)) c = (c + 31) / 32 * 32;
+    if (curk::ring_pays(dt, m, n)) {
+        c = (c + 31) / 32 * 32;
+        if (c < 128 && coltiles * ((m + 127) / 128) >= 3LL * num_sms) c = 128;
+    }
     *chunk = c;
     return (int)((m + c - 1) / c);
 }

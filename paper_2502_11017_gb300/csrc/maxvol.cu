@@ -1491,7 +1491,7 @@ static int rows_cap(int r, bool starts, bool kcta) {
     int lo = 1, hi = 1 << 20;
     while (lo < hi) {
         const int mid = (lo + hi + 1) / 2;
-        if ((kcta ? EngineSmem<TB>::bytes(mid, r, 0, true, false) : EngineSmem<TB>::bytes(mid, r, 0, false, r <= kMsMax)) <= smem_budget(r) &&
+        if ((kcta ? EngineSmem<TB>::bytes(mid, r, 0, true, false) : EngineSmem<TB>::bytes(mid, r, 0, false, r <= kMsMax)) <= (r > kMsMax && !kcta ? kEngineMost : smem_budget(r)) &&
             (!starts || StartSmem<TB>::bytes(mid, r) <= smem_budget(r))) lo = mid;
         else hi = mid - 1;
     }
@@ -1663,9 +1663,12 @@ template <typename TB>
 static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bool starts = false, bool may_start = false) {
     const int P = (int)sg.probs.size();
     sg.P = P;
+    // FP64 factorises C(S,:) every cycle and carries nothing between: a keeper CTA would stand idle
+    // (38 problems of 600 x 96: 190 CTAs where 152 do, 11.7 -> 13.3 ms)
+    constexpr bool keeps = !std::is_same<TB, double>::value;
     int capr[129] = {0};   // rows per CTA with B in shared memory, by rank
     auto cap_of = [&](int rr) {
-        if (!capr[rr]) capr[rr] = rows_cap<TB>(rr, starts || may_start || rr <= kMsMax, rr > kMsMax);
+        if (!capr[rr]) capr[rr] = rows_cap<TB>(rr, starts || may_start || rr <= kMsMax, keeps && rr > kMsMax);
         return capr[rr];
     };
     int64_t tot_p = 0;
@@ -1680,14 +1683,14 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
     for (auto& pr : sg.probs) {
         const int cap = cap_of(pr.r);
         int64_t G = (pr.p + cap - 1) / cap;
+        const int64_t share = (int64_t)h->num_sms * pr.p / std::max<int64_t>(1, tot_p);   // of the SMs
         pr.gmode = 0;
-        if (G > 1 && (many || G > h->num_sms - (pr.r > kMsMax)) && !starts) pr.gmode = 1;
+        if (G > 1 && (many || G > h->num_sms - (keeps && pr.r > kMsMax)) && !starts) pr.gmode = 1;
         if (pr.gmode && many) {
             G = 1;
         } else if (G > 1 || pr.gmode) {
             // spread large problems over the SMs in proportion to their size
-            const int64_t spread = std::min<int64_t>((pr.p + kSpreadRows - 1) / kSpreadRows,
-                                                     (int64_t)h->num_sms * pr.p / std::max<int64_t>(1, tot_p));
+            const int64_t spread = std::min<int64_t>((pr.p + kSpreadRows - 1) / kSpreadRows, share);
             G = std::max<int64_t>(pr.gmode ? 1 : G, spread);
             G = std::min<int64_t>(G, h->num_sms);
         }
@@ -1696,9 +1699,11 @@ static cur_status stage_setup(cur_handle* h, int r, Stage<TB>& sg, Arena& ar, bo
         // over the group's B in global memory would otherwise wait for the CTA that also
         // updates it
         pr.msm = pr.r <= kMsMax || EngineSmem<TB>::bytes((int)((pr.p + G - 1) / G), pr.r, pr.gmode ? EngineSmem<TB>::kStage : 0, false, true) <= smem_budget(pr.r);
-        pr.kcta = (!pr.msm && !(pr.gmode && many)) || (pr.gmode && G >= 8);
+        pr.kcta = pr.gmode ? (!pr.msm && !many) || G >= 8 : keeps && !pr.msm;
         if (!pr.gmode && (pr.p + cap - 1) / cap > h->num_sms - 1) pr.kcta = 0;   // no SM left for it
-        if (pr.kcta) {
+        if (pr.kcta) {   // out of the problem's share of the SMs: beside it, four problems of 3000 x 128 were 156 CTAs
+                         // and the last waited for the others (3.9 -> 5.1 ms)
+            G = std::min<int64_t>(G, std::max<int64_t>(pr.gmode ? 1 : (pr.p + cap - 1) / cap, share - 1));
             G = std::min<int64_t>(G, h->num_sms - 1);
             pr.msm = 1;
         }
@@ -1854,7 +1859,7 @@ static cur_status stage_launch(cur_handle* h, const TB* basis, int r, const cur_
     bool wide = false;   // groups with more threads: M^-1 above kMsMax or B in global memory
     for (const auto& pr : sg.probs) {
         sm_eng = std::max(sm_eng, EngineSmem<TB>::bytes(pr.rpc, pr.r, pr.gmode, pr.kcta != 0, pr.msm != 0));
-        wide |= pr.gmode != 0 || pr.kcta != 0;
+        wide |= pr.gmode != 0 || pr.kcta != 0 || (std::is_same<TB, double>::value && pr.r > kMsMax);
         sm_start = std::max(sm_start, StartSmem<TB>::bytes(pr.rpc, pr.r));
     }
     CUR_TRY(set_smem_attr(mv_engine<TB>, sm_eng));

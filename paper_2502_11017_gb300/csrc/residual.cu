@@ -481,7 +481,10 @@ __global__ void __launch_bounds__(256) residual_w2_k(const double* __restrict__ 
     }
 }
 
-template <typename TA>
+// WHOLE: m and n are multiples of the tile and A lies on pairs, so that the kernel has no code for ends and
+// keeps its registers for the sums: 262144 x 16384 BF16, r = 128, 21.9 ms, with ends 23.8; FP32
+// 65536 x 8192, r = 100, 2.44 and 2.60.
+template <typename TA, bool WHOLE>
 __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__ A, int64_t m, int64_t n, int64_t ld,
                                                           const TA* __restrict__ C, const float* __restrict__ W,
                                                           int64_t npad, int r, int64_t ntile_n, int64_t ntiles,
@@ -562,7 +565,7 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
             }
             if (kk < kc) step(x, y);
         }
-        const bool whole = pairs && c0 + kRfB <= n;
+        const bool whole = WHOLE || (pairs && c0 + kRfB <= n);
 #pragma unroll
         for (int grp = 0; grp < 2; ++grp) {
             float tmx = 0.f, tse = 0.f, tsa = 0.f;
@@ -576,7 +579,7 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
 #pragma unroll
             for (int a0 = 0; a0 < 8; a0 += 4) {
                 const int64_t i0 = r0 + ty * 16 + grp * 8 + a0;
-                if (whole && i0 + 4 <= m) {   // two elements per load, sixteen loads in flight
+                if (WHOLE || (whole && i0 + 4 <= m)) {   // two elements per load, sixteen loads in flight
                     uint64_t raw[4][4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
@@ -599,21 +602,22 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
                             const uint64_t d = acc[row >> 1][b];
                             fold(__uint_as_float(bits), __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)));
                         }
-                } else {
+                } else if constexpr (!WHOLE) {
                     // A's last rows or columns, or rows off the pairs' grid: one element per load, the
                     // 32 loads issued before they are folded, and an entry past A's end folds as zeros
                     // (loaded and folded one by one: BF16 113763 x 393, r = 16, 240 us; residual_k 169,
-                    // this 147). BF16 loads some valid address instead of a predicate: its conversions
-                    // otherwise wait for each load in turn (259 us); FP32 is faster with one (124 and 148)
+                    // this 136). BF16 loads some valid address instead of a predicate: its conversions
+                    // otherwise wait for each load in turn (228 us); FP32 is faster with one (119 and 148)
+                    const int rr = (int)min((int64_t)4, m - i0), rc = (int)min((int64_t)kRfB, n - c0);   // what A has here
                     TA raw[4][8];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
-                        const TA* p = A + min(i0 + a, m - 1) * ld;
+                        const TA* p = A + min(i0 + a, m - 1) * ld + c0;
 #pragma unroll
                         for (int b = 0; b < 8; ++b) {
-                            const int64_t col = c0 + 2 * tx + 32 * (b >> 1) + (b & 1);
-                            if constexpr (sizeof(TA) == 4) raw[a][b] = i0 + a < m && col < n ? p[col] : 0.f;
-                            else raw[a][b] = p[col < n ? col : 0];
+                            const int cc = 2 * tx + 32 * (b >> 1) + (b & 1);
+                            if constexpr (sizeof(TA) == 4) raw[a][b] = a < rr && cc < rc ? p[cc] : 0.f;
+                            else raw[a][b] = p[cc < rc ? cc : 0];
                         }
                     }
 #pragma unroll
@@ -622,7 +626,7 @@ __global__ void __launch_bounds__(kRfT, 2) residual_fma_k(const TA* __restrict__
                         for (int b = 0; b < 8; ++b) {
                             const int row = grp * 8 + a0 + a;
                             const uint64_t d = acc[row >> 1][b];
-                            const bool in = i0 + a < m && c0 + 2 * tx + 32 * (b >> 1) + (b & 1) < n;
+                            const bool in = a < rr && 2 * tx + 32 * (b >> 1) + (b & 1) < rc;
                             fold(in ? to_f(raw[a][b]) : 0.f, in ? __uint_as_float((uint32_t)(row & 1 ? d >> 32 : d)) : 0.f);
                         }
                 }
@@ -752,9 +756,10 @@ static cur_status residual_fma_t(cur_handle* h, const cur_mat* Am, const void* C
     CUR_CK(cudaGetLastError());
     note_launch();
     const size_t sm = (size_t)(2 * kRfKC + r) * kRfB * sizeof(float);
-    CUR_TRY(smem_attr((const void*)residual_fma_k<TA>, sm));
     const int pairs = (reinterpret_cast<uintptr_t>(Am->data) % (2 * sizeof(TA))) == 0 && Am->ld % 2 == 0;
-    residual_fma_k<TA><<<grid, kRfT, sm, st>>>(static_cast<const TA*>(Am->data), m, n, Am->ld, static_cast<const TA*>(C),
+    auto kernel = pairs && m % kRfB == 0 && n % kRfB == 0 ? residual_fma_k<TA, true> : residual_fma_k<TA, false>;
+    CUR_TRY(smem_attr((const void*)kernel, sm));
+    kernel<<<grid, kRfT, sm, st>>>(static_cast<const TA*>(Am->data), m, n, Am->ld, static_cast<const TA*>(C),
                                                W, npad, r, ntile_n, ntiles, part, pairs);
     CUR_CK(cudaGetLastError());
     note_launch();

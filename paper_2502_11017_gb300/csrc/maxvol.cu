@@ -1100,7 +1100,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) mv_engine(MvArgs a) {
     };
 
     // M^-1 is carried through the swaps by the first CTA, unless every cycle factorises C(S,:) afresh (FP64 data):
-    // then nothing reads it between (a cross of 2000 x 1500 FP64, r = 16: 2.74 -> 2.66 ms).
+    // then nothing reads it between.
     const bool carry = part == 0 && a.drift_max > 0.0;
     unsigned long long bk;   // argmax |B_ij| as an order key (coef_key), its flat index, a NaN seen
     long long bi;

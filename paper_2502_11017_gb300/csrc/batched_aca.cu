@@ -182,11 +182,11 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
 // batch above; 16-byte cp.async with a barrier per slot: 95.) What bounds it is the issue
 // slots: eleven FMA-pipe operations per element and about half as many instructions beside the packed sums. Words of the first
 // and last line that lie outside the matrix are not touched. `next` is the slot that fills
-// next and `phase` its parity. False: a copy did not arrive in time (`feed` false: none is made, for
+// next and `phase` its parity. False: a copy did not arrive in time (*feed 0: none is made, for
 // the self-test).
 template <bool DOT>
 __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m, int64_t n, int64_t ld, int cgn, int RG,
-                                         const df64* q, unsigned char* ring, int slot_b, bool feed, uint64_t* bars, uint64_t* freed,
+                                         const df64* q, unsigned char* ring, int slot_b, const int* feed, uint64_t* bars, uint64_t* freed,
                                          unsigned& next, unsigned& phase, df64* part) {
     const int tid = threadIdx.x, cg = tid % cgn, rg = tid / cgn;
     const bool active = rg < RG;
@@ -221,7 +221,7 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
                              :: "r"(su32(d + (lo - d0))), "l"(lo), "r"((uint32_t)(hi - lo)), "r"(su32(&bars[slot])) : "memory");
             }
         };
-        if (tid == 0 && feed)
+        if (tid == 0 && *feed)
             for (int s = 0; s < min(stages, kBA_Slots); ++s) fill(s, (next + s) % kBA_Slots);
         // addresses by addition only: the loop's issue slots are the sums'
         const int step = RG * (int)(ld * 4), first = active ? rg * (int)(ld * 4) : 0, bytes = per * (int)(ld * 4);
@@ -306,9 +306,9 @@ __device__ __forceinline__ bool bat_pass(const float* __restrict__ A, int64_t m,
 
 // order: the matrices by decreasing cost (r m n); queue: a zeroed counter. A CTA takes
 // the next matrix of the order when it finishes one (largest first, so the tail is short). A CTA
-// whose wait ran out records it and goes on through the queue without picks: counts and J hold valid
-// entries or -1 for every matrix whatever happens, and the padding and the gathers that follow rely
-// on that. drop: the matrix whose copies are withheld, `count` for all of them, < 0 for none.
+// whose wait ran out records it and ends its matrix and what is left of the queue without picks: counts
+// and J hold valid entries or -1 for every matrix whatever happens, and the padding and the gathers that
+// follow rely on that. drop: the matrix whose copies are withheld, `count` for all of them, < 0 for none.
 __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ data, const BatAcaItem* items,
                                                        const int32_t* order, int* queue, int count, int32_t* J,
                                                        int32_t* counts, float* Qws, int slot_b, int drop, int* status) {
@@ -319,12 +319,11 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
     df64* qs = v + kBA_MaxM;                                             // r
     unsigned char* mask = reinterpret_cast<unsigned char*>(qs + kBA_MaxR);
     __shared__ double s_frob2;
-    __shared__ int s_next;
+    __shared__ int s_next, s_feed;
     unsigned char* ring = mask + kBA_MaxN;
     __shared__ __align__(8) uint64_t bars[kBA_Slots], freed[kBA_Slots];
     const int tid = threadIdx.x;
     unsigned next = 0, phase = 0;
-    bool lost = false;   // a wait ran out (every thread alike)
     if (tid == 0) {
         for (int s = 0; s < kBA_Slots; ++s) {
             mbar_init(&bars[s], 1);
@@ -356,14 +355,23 @@ __global__ void __launch_bounds__(kBA_T, 2) bat_aca_k(const float* __restrict__ 
         const int RG = max(1, min((int)blockDim.x / cgn, (int)(kBA_RG * kBA_MaxN / n)));
         for (int j = tid; j < n; j += blockDim.x) mask[j] = 0;
         int picked = 0, bad = 0;
-        const bool feed = drop < 0 || (drop < count && drop != it);
-        for (int t = -1; t < r - 1 && !lost; ++t) {
+        if (tid == 0) s_feed = drop < 0 || (drop < count && drop != it);
+        for (int t = -1; t < r - 1; ++t) {
             // ---- pass: squared norms (t = -1) or w = A^T q_t
-            if (!(t < 0 ? bat_pass<false>(A, m, n, ld, cgn, RG, v, ring, slot_b, feed, bars, freed, next, phase, part)
-                        : bat_pass<true>(A, m, n, ld, cgn, RG, v, ring, slot_b, feed, bars, freed, next, phase, part))) {
+            if (!(t < 0 ? bat_pass<false>(A, m, n, ld, cgn, RG, v, ring, slot_b, &s_feed, bars, freed, next, phase, part)
+                        : bat_pass<true>(A, m, n, ld, cgn, RG, v, ring, slot_b, &s_feed, bars, freed, next, phase, part))) {
+                if (tid != 0) return;
                 set_status(status, CUR_ERR_TIMEOUT);
-                lost = true;
-                break;
+                int end = it, k0 = picked;
+                while (true) {
+                    const BatAcaItem e = items[end];
+                    counts[end] = k0;
+                    for (int k = k0; k < e.r; ++k) J[e.joff + k] = -1;
+                    const int at = atomicAdd(queue, 1);
+                    if (at >= count) return;
+                    end = order[at];
+                    k0 = 0;
+                }
             }
             // ---- pick
             unsigned long long bk = dkey(-INFINITY);
